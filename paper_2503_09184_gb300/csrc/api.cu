@@ -86,9 +86,9 @@ struct sfhe_ctx {
     u64* d_s;
     signed char* d_s_coeff;
     u64* d_rlk;     // the key, followed in the same allocation by
-    u64* d_rlk_sh;  // its Shoup companions
+    u64* d_rlk_pm;  // the key in pm_mul's form (twice its words)
     int* d_err;
-    // persisting-L2 window over the key and companions (bytes 0: none)
+    // persisting-L2 window over the key in pm_mul's form (bytes 0: none)
     size_t l2_bytes;
     float l2_hit;
     // tile tuning of the per-product persistent kernel
@@ -166,7 +166,7 @@ extern "C" sfhe_status sfhe_cdt_table(double sigma, uint64_t* T20)
 
 // ---------------------------------------------------------------- context ---
 // Stage R reads the whole key once per output entry.  A persisting
-// access-policy window over the key and its companions keeps them in L2
+// access-policy window over the key (pm_mul's form) keeps it in L2
 // between entries while the per-product scratch streams through: the
 // context raises its persisting-L2 limit (a limit of this process's
 // context, released with it) to the key's size or the device's maximum,
@@ -205,7 +205,7 @@ extern "C" void sfhe_ctx_destroy(sfhe_ctx* c)
     cudaFree(c->d_twb);
     cudaFree(c->d_s);
     cudaFree(c->d_s_coeff);
-    cudaFree(c->d_rlk);  // the companions share the allocation
+    cudaFree(c->d_rlk);  // both forms share the allocation
     cudaFree(c->d_err);
     delete c;
 }
@@ -249,7 +249,7 @@ extern "C" sfhe_status sfhe_ctx_create(const sfhe_params* params, uint64_t seed,
     cdt_table(params->sigma, rc.cdt);
 
     std::vector<uint64_t> tw((size_t)rc.L * 4 * N);
-    for (int i = 0; i < rc.L; i++) twiddles(rc.m[i].q, N, tw.data() + (size_t)i * 4 * N, &rc.ninv[i], &rc.wlast[i]);
+    for (int i = 0; i < rc.L; i++) twiddles_pm(rc.m[i].q, N, tw.data() + (size_t)i * 4 * N, &rc.ninv_pm[i], &rc.wlast_pm[i]);
     std::vector<uint32_t> twb((size_t)rc.K * 4 * N);
     for (int k = 0; k < rc.K; k++)
         twiddles32(rc.mb[k].b, N, twb.data() + (size_t)k * 4 * N, &rc.ninv_b[k], &rc.wlast_b[k]);
@@ -258,17 +258,17 @@ extern "C" sfhe_status sfhe_ctx_create(const sfhe_params* params, uint64_t seed,
     const size_t rlk_words = (size_t)L * 2 * L * N;
     if (cudaMalloc(&c->d_tw, tw.size() * 8) != cudaSuccess || cudaMalloc(&c->d_twb, twb.size() * 4) != cudaSuccess ||
         cudaMalloc(&c->d_s, (size_t)L * N * 8) != cudaSuccess ||
-        cudaMalloc(&c->d_s_coeff, N) != cudaSuccess || cudaMalloc(&c->d_rlk, 2 * rlk_words * 8) != cudaSuccess ||
+        cudaMalloc(&c->d_s_coeff, N) != cudaSuccess || cudaMalloc(&c->d_rlk, 3 * rlk_words * 8) != cudaSuccess ||
         cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess)
         return bail(fail(SFHE_ENOMEM, "device allocation of the context failed"));
-    c->d_rlk_sh = c->d_rlk + rlk_words;
+    c->d_rlk_pm = c->d_rlk + rlk_words;
     rc.tw = c->d_tw;
     rc.twb = c->d_twb;
     if (cudaMemcpy(c->d_tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->d_twb, twb.data(), twb.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess)
         return bail(fail(SFHE_ECUDA, "table upload failed"));
-    cudaError_t e = launch_keygen(rc, c->d_s, c->d_s_coeff, c->d_rlk, c->d_rlk_sh, c->d_err, 0);
+    cudaError_t e = launch_keygen(rc, c->d_s, c->d_s_coeff, c->d_rlk, c->d_rlk_pm, c->d_err, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return bail(fail(SFHE_ECUDA, "key generation: %s", cudaGetErrorString(e)));
     int err = 0;
@@ -737,8 +737,7 @@ PersistentArgs persistent_args(const sfhe_plan* P, int n_entries, int variant)
     a.entries = P->d_entries;
     a.n_entries = n_entries;
     a.rowlist = P->d_rowlist;
-    a.rlk = c->d_rlk;
-    a.rlk_sh = c->d_rlk_sh;
+    a.rlk = c->d_rlk_pm;
     a.scratch = P->d_scratch;
     a.scratch_stride = P->scratch_stride;
     a.queue = P->d_queue;
@@ -746,7 +745,7 @@ PersistentArgs persistent_args(const sfhe_plan* P, int n_entries, int variant)
     a.grid = P->grid;
     a.grouped = (P->flags & SFHE_EXEC_LAZY) != 0;
     a.variant = a.grouped ? 0 : variant;
-    a.l2_base = c->d_rlk;
+    a.l2_base = c->d_rlk_pm;
     a.l2_bytes = c->l2_bytes;
     a.l2_hit_ratio = c->l2_hit;
     return a;
@@ -831,7 +830,7 @@ sfhe_status launch_plan(sfhe_plan* P, cudaStream_t s)
             CUDA_TRY(launch_tensor_intt(rc, a, b, P->d_T, s));
             CUDA_TRY(launch_scale_round(rc, P->d_T, P->d_D, s));
             CUDA_TRY(launch_relin_ntt(rc, P->d_D, P->d_U, s));
-            CUDA_TRY(launch_relin_accum(rc, P->d_U, c->d_rlk, c->d_rlk_sh, Cout, s));
+            CUDA_TRY(launch_relin_accum(rc, P->d_U, c->d_rlk_pm, Cout, s));
         }
     }
     return SFHE_OK;
@@ -1194,7 +1193,7 @@ extern "C" sfhe_status sfhe_ct_mul_relin(sfhe_ctx* c, const uint32_t* a_ext, con
     CUDA_TRY(launch_tensor_intt(c->rc, a_ext, b_ext, T, s));
     CUDA_TRY(launch_scale_round(c->rc, T, D, s));
     CUDA_TRY(launch_relin_ntt(c->rc, D, U, s));
-    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk, c->d_rlk_sh, out, s));
+    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, s));
     return SFHE_OK;
 }
 
@@ -1231,7 +1230,7 @@ extern "C" sfhe_status sfhe_ct_mul_relin_static(sfhe_ctx* c, const uint32_t* a_e
     CUDA_TRY(launch_tensor_intt(c->rc, a_ext, b_ext, T, s));
     CUDA_TRY(launch_scale_round(c->rc, T, D, s));
     CUDA_TRY(launch_relin_ntt(c->rc, D, U, s));
-    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk, c->d_rlk_sh, out, s));
+    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, s));
     return SFHE_OK;
 }
 

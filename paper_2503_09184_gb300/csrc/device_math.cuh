@@ -64,6 +64,70 @@ SFHE_DEV u64 barrett_lazy(u64 hi, u64 lo, Mod m)
     return lo - mulhi(xs, m.mu) * m.q;
 }
 
+// ------------------------------------------------ q = 2^54 - c arithmetic ---
+// The ciphertext primes are the largest below 2^54 that are 1 mod 2N, so
+// c = 2^54 - q is small (below 2^22.4 in every supported ring; the host
+// checks c < 2^23) and 2^54 = c mod q: a value folds by one 32-bit multiply
+// instead of a quotient estimate.  Values are signed 64-bit words.
+typedef long long i64;
+SFHE_DEV int pm_c(u64 q) { return (int)(0u - (u32)q); }
+
+// a w mod q for |a| <= 2^62 and a prepared constant (w, w2): with
+// a = a1 2^32 + a0 (a0 signed), a w = a0 w + a1 (2^32 w), and with the
+// constants split at bit 22 the sum is p0 + 2^22 p1 = p0 + 2^22 lo(p1) +
+// 2^54 hi(p1), whose last term folds to c hi(p1): five signed 32x32->64-bit
+// multiply-adds, no carries (Shoup's form of the same product takes ten
+// 32-bit multiplies and their carries).  |p1| < 2^62 + 2^61,
+// |p0| < 2^53 + 2^52; the result lies in (-2^54.6, 2^55.3) for any such a,
+// and within 2^55 for |a| <= 2^60.  A 32x32->64-bit multiply-add occupies
+// the issue of a scheduler for 4.25 cycles (measured, full chip), a 32-bit
+// one or a shift for 2.1, an add for 1.06: the product costs 26 cycles per
+// warp, Shoup's 34.  (Written with inline PTX: from C++ the signed products
+// were compiled to 47 cycles.)
+SFHE_DEV i64 mad_wide(int a, int b, i64 c)
+{
+    i64 d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+SFHE_DEV i64 mul_wide(int a, int b)
+{
+    i64 d;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+}
+SFHE_DEV i64 pm_mul(i64 a, u64 w, u64 w2, int c)
+{
+    const int a0 = (int)a, a1 = (int)(a >> 32) + (int)((u32)a0 >> 31);
+    const i64 p1 = mad_wide(a1, (int)(w2 >> 32), mul_wide(a0, (int)(w >> 32)));
+    const i64 p0 = mad_wide(a1, (int)w2, mul_wide(a0, (int)w));
+    return mad_wide((int)(p1 >> 32), c, p0) + (i64)((u64)(u32)p1 << 22);
+}
+// one fold: v mod q in (-2^33, 2^54 + 2^33) for any signed 64-bit v
+SFHE_DEV i64 pm_fold(i64 v, int c)
+{
+    const int h = (int)(v >> 54);
+    return mad_wide(h, c, (i64)((u64)v & ((1ULL << 54) - 1)));
+}
+// the same for an unsigned word: below 2^54 + 2^33
+SFHE_DEV i64 pm_fold_u(u64 v, int c)
+{
+    return mad_wide((int)(u32)(v >> 54), c, (i64)(v & ((1ULL << 54) - 1)));
+}
+// canonical residue of any signed 64-bit v
+SFHE_DEV u64 pm_canon(i64 v, u64 q)
+{
+    i64 r = pm_fold(v, pm_c(q));
+    r += r < 0 ? (i64)q : 0;
+    return r >= (i64)q ? (u64)r - q : (u64)r;
+}
+// the constant's two packed words from its canonical residue
+SFHE_DEV u64 pm_pack(u64 w, u64 q)
+{
+    const i64 s = w > q / 2 ? (i64)w - (i64)q : (i64)w;
+    return ((u64)(u32)(int)(s >> 22) << 32) | ((u64)s & ((1u << 22) - 1));
+}
+
 // (hi:lo) += a * b
 SFHE_DEV void mac(u64& hi, u64& lo, u64 a, u64 b)
 {

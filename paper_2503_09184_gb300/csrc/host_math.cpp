@@ -249,6 +249,46 @@ void twiddles(uint64_t q, uint32_t N, uint64_t* out, ShoupC* ninv, ShoupC* wlast
     *wlast = shoup_of(mulm(g[1], ni, q), q);
 }
 
+static uint64_t pm_pack(uint64_t w, uint64_t q)
+{
+    const int64_t s = w > q / 2 ? (int64_t)w - (int64_t)q : (int64_t)w;
+    const int64_t lo = s & ((1 << 22) - 1);  // floor remainder
+    return ((uint64_t)(uint32_t)(int32_t)((s - lo) / (1 << 22)) << 32) | (uint64_t)lo;
+}
+
+PmC pm_of(uint64_t w, uint64_t q)
+{
+    PmC c;
+    c.w = pm_pack(w, q);
+    c.w2 = pm_pack(mulm(w, 1ULL << 32, q), q);
+    return c;
+}
+
+void twiddles_pm(uint64_t q, uint32_t N, uint64_t* out, PmC* ninv, PmC* wlast)
+{
+    std::vector<uint64_t> f, g;
+    root_tables(q, N, f, g);
+    const uint32_t nt = N / 16;  // threads of the transform
+    for (uint32_t k = 0; k < N; ++k) {
+        // levels of the pass on runs of 16 elements: lane-interleaved
+        uint32_t at = k;
+        if (k >= nt) {
+            uint32_t base = nt;
+            while (2 * base <= k) base *= 2;
+            const uint32_t c = base / nt, r = k - base;
+            at = base + (r % c) * nt + r / c;
+        }
+        const PmC a = pm_of(f[k], q), b = pm_of(g[k], q);
+        out[2 * at] = a.w;
+        out[2 * at + 1] = a.w2;
+        out[2 * N + 2 * at] = b.w;
+        out[2 * N + 2 * at + 1] = b.w2;
+    }
+    const uint64_t ni = invm(N, q);
+    *ninv = pm_of(ni, q);
+    *wlast = pm_of(mulm(g[1], ni, q), q);
+}
+
 void twiddles32(uint32_t b, uint32_t N, uint32_t* out, Shoup32* ninv, Shoup32* wlast)
 {
     std::vector<uint64_t> f, g;
@@ -350,6 +390,11 @@ static uint64_t prod_b(const RnsConsts& rc, int count, int skip, uint64_t m)
 bool fill_constants(RnsConsts& rc)
 {
     const int L = rc.L, K = rc.K;
+    for (int i = 0; i < L; ++i) {
+        // pm_mul's range analysis: q = 2^54 - c, c < 2^23
+        if (rc.m[i].q >> 54 || (1ULL << 54) - rc.m[i].q >= (1ULL << 23)) return false;
+        rc.ninv[i] = shoup_of(invm(rc.N, rc.m[i].q), rc.m[i].q);
+    }
     const uint64_t t = rc.t;
     // exact size margin: B > 2 N Q^2 (the centred tensor |x| < N Q^2 / 2)
     Big Qbig = big(1), Bbig = big(1);

@@ -25,6 +25,11 @@ void cdt_table(double sigma, uint64_t* T);
 // 64-bit version is for the 54-bit primes (Shoup companions over 2^64), the
 // 32-bit one for the 30-bit primes (companions over 2^32).
 void twiddles(uint64_t q, uint32_t N, uint64_t* out4N, ShoupC* ninv, ShoupC* wlast);
+// The same for q = 2^54 - c in pm_mul's form: [2][N] pairs (PmC), of psi_rev
+// and of ipsi_rev, the levels of the pass on runs of 16 elements
+// lane-interleaved (NttT::tw_pair).
+void twiddles_pm(uint64_t q, uint32_t N, uint64_t* out4N, PmC* ninv, PmC* wlast);
+PmC pm_of(uint64_t w, uint64_t q);
 void twiddles32(uint32_t b, uint32_t N, uint32_t* out4N, Shoup32* ninv, Shoup32* wlast);
 // Fills every base-conversion constant of rc from its primes (rc.m[].q,
 // rc.mb[].b, rc.L, rc.K, rc.t, rc.N set).  Returns false if a size

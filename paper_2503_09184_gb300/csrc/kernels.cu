@@ -136,7 +136,7 @@ cudaError_t launch_ntt32(const RnsConsts& rc, bool inverse, const u32* in, size_
 }
 
 template <int LOGN>
-static cudaError_t keygen_impl(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_sh, int* err,
+static cudaError_t keygen_impl(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_pm, int* err,
                                cudaStream_t s)
 {
     const size_t smem = smem_of<LOGN>();
@@ -145,14 +145,14 @@ static cudaError_t keygen_impl(const RnsConsts& rc, u64* s_ntt, signed char* s_c
     if (e != cudaSuccess) return e;
     k_keygen_secret<LOGN><<<rc.L, nt_of<LOGN>(), smem, s>>>(rc, s_ntt, s_coeff, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_keygen_rlk<LOGN><<<dim3(rc.L, rc.L), nt_of<LOGN>(), smem, s>>>(rc, s_ntt, rlk, rlk_sh, err);
+    k_keygen_rlk<LOGN><<<dim3(rc.L, rc.L), nt_of<LOGN>(), smem, s>>>(rc, s_ntt, rlk, rlk_pm, err);
     return cudaGetLastError();
 }
 
-cudaError_t launch_keygen(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_sh, int* err,
+cudaError_t launch_keygen(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_pm, int* err,
                           cudaStream_t s)
 {
-    SFHE_DISPATCH_LOGN(rc.logN, return keygen_impl<LG>(rc, s_ntt, s_coeff, rlk, rlk_sh, err, s));
+    SFHE_DISPATCH_LOGN(rc.logN, return keygen_impl<LG>(rc, s_ntt, s_coeff, rlk, rlk_pm, err, s));
 }
 
 template <int LOGN>
@@ -226,10 +226,9 @@ cudaError_t launch_relin_ntt(const RnsConsts& rc, const u64* D, u64* U, cudaStre
     });
 }
 
-cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk, const u64* rlk_sh, u64* C,
-                               cudaStream_t s)
+cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, cudaStream_t s)
 {
-    k_relin_accum<<<dim3((rc.N + 255) / 256, rc.L), 256, 0, s>>>(rc, U, rlk, rlk_sh, C);
+    k_relin_accum<<<dim3((rc.N + 255) / 256, rc.L), 256, 0, s>>>(rc, U, rlk_pm, C);
     return cudaGetLastError();
 }
 

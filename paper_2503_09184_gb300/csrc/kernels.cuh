@@ -3,7 +3,7 @@
 // Storage (canonical residues):
 //   ciphertext, base Q, NTT form:          [2 (c0, c1)][L][N]  uint64
 //   lifted ciphertext, base B, NTT form:   [2][K][N]           uint32 (lane-interleaved, NttT::lane_idx)
-//   relinearisation key, base Q, NTT form: [L digit j][2 (b, a)][L limb i][N] uint64 (+ Shoup companions)
+//   relinearisation key, base Q, NTT form: [L digit j][2 (b, a)][L limb i][N] uint64 (canonical; and in pm_mul's form)
 // Per product (Alg. 1's inner loop: multiply, relinearise, add):
 //   tensor d0 = a0 b0, d1 = a0 b1 + a1 b0, d2 = a1 b1 over B (NTT form, 30-bit
 //   arithmetic), inverse NTT: the exact integer tensor x in B (|x| < B / 4);
@@ -237,6 +237,12 @@ SFHE_DEV void scale_round_b(const u32* x32, size_t stride, const RnsConsts& c, u
 // ------------------------------------------------------------------------
 // generic NTT kernels over batches of polynomials
 // ------------------------------------------------------------------------
+// Over Q the kernel issues integer multiplies (five 32x32->64-bit ones per
+// butterfly, which do not overlap with other issues) and shared-memory
+// exchanges; global words are read and written coalesced through one more
+// exchange.  4096 transforms at N = 8192, L = 4 (GB300): inverse 477 -> 300
+// us, forward 451 -> 316 us against Shoup butterflies with run-layout
+// accesses; at N = 16384, L = 8 (16384 transforms) 1956 -> 1200 us.
 // Polynomial (g, l): input at in + g * in_gstride + (in_l0 + l) * N, output
 // at out + g * out_gstride + (out_l0 + l) * N, prime index prime0 + l of Q.
 template <int LOGN>
@@ -252,10 +258,13 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_ntt_fwd(const __grid_c
     u64* dst = out + g * out_gstride + (size_t)(out_l0 + l) * NT_::N;
     u64 x[NT_::R];
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::fwd_in_idx(v, tid)];
+    for (int v = 0; v < NT_::R; v++) x[v] = (u64)pm_fold_u(src[NT_::fwd_in_idx(v, tid)], pm_c(m.q));
     NT_::forward(x, sm, tid, c.tw + (size_t)pi * 4 * NT_::N, m.q);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) dst[NT_::run_idx(v, tid)] = barrett64(x[v], m);
+    for (int v = 0; v < NT_::R; v++) x[v] = pm_canon((i64)x[v], m.q);
+    NT_::run_to_lane(x, sm, tid);
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = x[v];
 }
 
 template <int LOGN>
@@ -271,11 +280,12 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_ntt_inv(const __grid_c
     u64* dst = out + g * out_gstride + (size_t)(out_l0 + l) * NT_::N;
     u64 x[NT_::R];
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) x[v] = csub(src[NT_::run_idx(v, tid)], m.q);
-    NT_::inverse(x, sm, tid, c.tw + (size_t)pi * 4 * NT_::N, m.q, c.ninv[pi].w, c.ninv[pi].ws, c.wlast[pi].w,
-                 c.wlast[pi].ws);
+    for (int v = 0; v < NT_::R; v++) x[v] = (u64)pm_fold_u(src[NT_::lane_idx(v, tid)], pm_c(m.q));
+    NT_::lane_to_run(x, sm, tid);
+    NT_::inverse(x, sm, tid, c.tw + (size_t)pi * 4 * NT_::N, m.q, c.ninv_pm[pi].w, c.ninv_pm[pi].w2, c.wlast_pm[pi].w,
+                 c.wlast_pm[pi].w2);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) dst[NT_::inv_out_idx(v, tid)] = csub(x[v], m.q);
+    for (int v = 0; v < NT_::R; v++) dst[NT_::inv_out_idx(v, tid)] = pm_canon((i64)x[v], m.q);
 }
 
 // Same over the tensor base (32-bit words, prime index into B).
@@ -349,17 +359,21 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_keygen_secret(const __
         x[v] = to_residue(s, m.q);
     }
     NT_::forward(x, sm, tid, c.tw + (size_t)l * 4 * NT_::N, m.q);
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) s_ntt[(size_t)l * NT_::N + NT_::run_idx(v, tid)] = barrett64(x[v], m);
+    for (int v = 0; v < NT_::R; v++) s_ntt[(size_t)l * NT_::N + NT_::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
     if (fail) atomicExch(err, 1);
 }
 
 // Relinearisation key, block (i limb, j digit):
 //   a uniform (coefficient form, NTT'd), e_j Gaussian,
-//   b = -a s + e_j + delta_ij s^2  (NTT form), plus Shoup companions.
+//   b = -a s + e_j + delta_ij s^2  (NTT form); rlk_pm: the same words in
+//   pm_mul's form, [L][2][L][N] pairs (w, w2), each polynomial's pairs
+//   lane-interleaved (NttT::lane_idx), as the transforms that multiply by
+//   them hold their output.
 template <int LOGN>
 __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_keygen_rlk(const __grid_constant__ RnsConsts c, const u64* s_ntt,
-                                                                    u64* rlk, u64* rlk_sh, int* err)
+                                                                    u64* rlk, u64* rlk_pm, int* err)
 {
     using NT_ = typename NttGeom<LOGN>::T;
     constexpr int N = NT_::N;
@@ -381,19 +395,20 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_keygen_rlk(const __gri
     NT_::forward(e, sm, tid, tw, m.q);
     u64* b_out = rlk + (((size_t)j * 2 + 0) * L + i) * N;
     u64* a_out = rlk + (((size_t)j * 2 + 1) * L + i) * N;
-    u64* bs_out = rlk_sh + (((size_t)j * 2 + 0) * L + i) * N;
-    u64* as_out = rlk_sh + (((size_t)j * 2 + 1) * L + i) * N;
+    ulonglong2* bp_out = reinterpret_cast<ulonglong2*>(rlk_pm) + (((size_t)j * 2 + 0) * L + i) * N;
+    ulonglong2* ap_out = reinterpret_cast<ulonglong2*>(rlk_pm) + (((size_t)j * 2 + 1) * L + i) * N;
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::run_idx(v, tid);
-        const u64 av = barrett64(a[v], m), ev = barrett64(e[v], m);
+        const u64 av = pm_canon((i64)a[v], m.q), ev = pm_canon((i64)e[v], m.q);
         const u64 sv = s_ntt[(size_t)i * N + k];
         u64 bv = sub_mod(ev, mul_mod(av, sv, m), m.q);
         if (i == j) bv = add_mod(bv, mul_mod(sv, sv, m), m.q);
         b_out[k] = bv;
         a_out[k] = av;
-        bs_out[k] = (u64)(((unsigned __int128)bv << 64) / m.q);
-        as_out[k] = (u64)(((unsigned __int128)av << 64) / m.q);
+        const int kl = NT_::lane_idx(v, tid);
+        bp_out[kl] = make_ulonglong2(pm_pack(bv, m.q), pm_pack(barrett(bv >> 32, bv << 32, m), m.q));
+        ap_out[kl] = make_ulonglong2(pm_pack(av, m.q), pm_pack(barrett(av >> 32, av << 32, m), m.q));
     }
     if (fail) atomicExch(err, 1);
 }
@@ -431,11 +446,13 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_encrypt(const __grid_c
     NT_::forward(e, sm, tid, tw, m.q);
     u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
     u64* c1 = c0 + (size_t)L * N;
+    NT_::run_to_lane(a, sm, tid);
+    NT_::run_to_lane(e, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
-        const int k = NT_::run_idx(v, tid);
-        const u64 av = barrett64(a[v], m);
-        c0[k] = sub_mod(barrett64(e[v], m), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
+        const int k = NT_::lane_idx(v, tid);
+        const u64 av = pm_canon((i64)a[v], m.q);
+        c0[k] = sub_mod(pm_canon((i64)e[v], m.q), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
         c1[k] = av;
     }
     if (fail) atomicExch(err, 1);
@@ -566,7 +583,8 @@ __global__ void __launch_bounds__(128) k_scale_round(const __grid_constant__ Rns
 }
 
 // block (target limb i, source s): s = 0: d0_i, 1: d1_i, 2+j: [D_j]_{q_i}
-// (digit j = d2 mod q_j); forward NTT into U[s][i][N]
+// (digit j = d2 mod q_j); forward NTT into U[s][i][N] (signed lazy words,
+// lane-interleaved)
 template <int LOGN>
 __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_relin_ntt(const __grid_constant__ RnsConsts c, const u64* D,
                                                                    u64* U)
@@ -579,30 +597,33 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_relin_ntt(const __grid
     const u64* src = s == 0 ? D + (size_t)i * N : (s == 1 ? D + ((size_t)L + i) * N : D + ((size_t)2 * L + (s - 2)) * N);
     u64 x[NT_::R];
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::fwd_in_idx(v, tid)];  // < 2^54: fine as lazy input
+    for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::fwd_in_idx(v, tid)];  // < 2^54: a valid forward input
     NT_::forward(x, sm, tid, c.tw + (size_t)i * 4 * N, m.q);
     u64* dst = U + ((size_t)s * L + i) * N;
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) dst[NT_::run_idx(v, tid)] = barrett64(x[v], m);
+    for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = x[v];
 }
 
 #ifdef SFHE_KERNELS_TU
-// C[p][i] += U[p][i] + sum_j U[2+j][i] rlk[j][p][i]   (p = 0: b, 1: a)
-__global__ void __launch_bounds__(256) k_relin_accum(const __grid_constant__ RnsConsts c, const u64* U, const u64* rlk,
-                                                     const u64* rlk_sh, u64* C)
+// C[p][i] += U[p][i] + sum_j U[2+j][i] rlk[j][p][i]   (p = 0: b, 1: a); U and
+// the key lane-interleaved, R = 16 words per thread of the transform
+__global__ void __launch_bounds__(256) k_relin_accum(const __grid_constant__ RnsConsts c, const u64* U, const u64* rlk_pm,
+                                                     u64* C)
 {
     const int N = c.N, L = c.L;
     const int k = blockIdx.x * 256 + threadIdx.x, i = blockIdx.y;
     if (k >= N) return;
     const Mod m = c.m[i];
+    const int pc = pm_c(m.q);
+    const int nt = N / 16, e = (k % nt) * 16 + k / nt;  // the slot stored at k
     for (int p = 0; p < 2; p++) {
-        u64 acc = U[((size_t)p * L + i) * N + k];
+        i64 acc = (i64)U[((size_t)p * L + i) * N + k];
         for (int j = 0; j < L; j++) {
-            const size_t ro = (((size_t)j * 2 + p) * L + i) * N + k;
-            acc += shoup_lazy(U[((size_t)(2 + j) * L + i) * N + k], rlk[ro], rlk_sh[ro], m.q);
+            const ulonglong2 w = reinterpret_cast<const ulonglong2*>(rlk_pm)[(((size_t)j * 2 + p) * L + i) * N + k];
+            acc += pm_mul((i64)U[((size_t)(2 + j) * L + i) * N + k], w.x, w.y, pc);
         }
-        u64* cp = C + ((size_t)p * L + i) * N + k;
-        *cp = add_mod(*cp, barrett64(acc, m), m.q);
+        u64* cp = C + ((size_t)p * L + i) * N + e;
+        *cp = add_mod(*cp, pm_canon(acc, m.q), m.q);
     }
 }
 
@@ -682,17 +703,18 @@ struct PersistentTile {
 // bulk copy did not complete within the wait bound).  mbarriers 0 and 1
 // track the operand pairs of stage T.
 template <int LOGN, int L, bool GROUPED, int V>
-__global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_matmul_persistent(
+__global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
     const __grid_constant__ RnsConsts c, const MmDesc* __restrict__ mms, const Entry* __restrict__ entries, int n_entries,
-    const int2* __restrict__ rowlist, const u64* __restrict__ rlk, const u64* __restrict__ rlk_sh, u64* scratch,
+    const int2* __restrict__ rowlist, const u64* __restrict__ rlk, u64* scratch,
     size_t scratch_stride, unsigned* queue, const unsigned* stop)
 {
     using CF = Cfg<LOGN, L>;
     using NQ = typename CF::NQ;
     using NB = typename PersistentTile<LOGN, L, V>::NB;
     using PP = PersistentPlan<LOGN, L>;
-    static_assert(NQ::NT == NB::NT, "both transforms use the same CTA");
-    constexpr int N = NQ::N, NTH = NQ::NT, K = CF::K, R = NB::R;
+    constexpr int N = NQ::N, NTH = NB::NT, K = CF::K, R = NB::R;
+    constexpr int VT = NQ::NT / NTH;  // virtual threads of the 64-bit transforms per thread
+    static_assert(VT == (PP::STAGED ? 1 : VT), "one virtual thread per thread up to N = 8192");
     extern __shared__ __align__(128) u64 sm[];
     u32* sm32 = reinterpret_cast<u32*>(sm);
     unsigned char* smb = reinterpret_cast<unsigned char*>(sm);
@@ -705,6 +727,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_matmul_persistent(
     u32* T = reinterpret_cast<u32*>(cacc + (size_t)2 * N);  // [3][K][N] u32
     const size_t ext_words = (size_t)2 * K * N;
     const size_t ct_words = (size_t)2 * L * N;
+    const ulonglong2* key = reinterpret_cast<const ulonglong2*>(rlk);  // pairs, lane-interleaved
     // staged operand slots: 0 a0, 1 a1, 2 b0, 3 b1 (limb k of the tensor base)
     auto slot = [&](int s) { return reinterpret_cast<u32*>(smb + PP::EXB + (size_t)s * PP::SLOT); };
     // per mbarrier: parity of the phase to wait for next, and whether a copy
@@ -1191,101 +1214,87 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_matmul_persistent(
         // N = 16384 they do not fit: the L + 2 transforms of a limb go to the
         // idle tensor scratch and one pass forms both sums in registers.
         if constexpr (PP::STAGED) {
-            u64* cs = PP::STAGED ? reinterpret_cast<u64*>(smb + PP::EXB) : cacc;
-            auto cpos = [&](int v) -> size_t {
-                return PP::STAGED ? (size_t)v * NTH + tid : (size_t)NQ::run_idx(v, tid);
-            };
+            u64* cs = reinterpret_cast<u64*>(smb + PP::EXB);
             for (int i = 0; i < L; i++) {
                 const Mod m = c.m[i];
+                const int pc = pm_c(m.q);
                 const u64* tw = c.tw + (size_t)i * 4 * N;
                 for (int s = 0; s < L + 2; s++) {
                     // s = 0: sum d0 (limb i), 1: sum d1 (limb i), 2 + j: sum of digits j
                     const u64* src = s < 2 ? acc + ((size_t)s * L + i) * N : acc + ((size_t)2 * L + (s - 2)) * N;
                     u64 x[NQ::R];
 #pragma unroll
-                    for (int v = 0; v < NQ::R; v++) x[v] = barrett64(src[NQ::fwd_in_idx(v, tid)], m);
+                    for (int v = 0; v < NQ::R; v++) x[v] = (u64)pm_fold_u(src[NQ::fwd_in_idx(v, tid)], pc);
                     NQ::forward(x, sm, tid, tw, m.q);
                     if (s < 2) {
 #pragma unroll
-                        for (int v = 0; v < NQ::R; v++) cs[(size_t)s * N + cpos(v)] = x[v];
+                        for (int v = 0; v < NQ::R; v++) cs[(size_t)s * N + NQ::lane_idx(v, tid)] = x[v];
                     } else {
                         const int j = s - 2;
-                        const size_t ob = (((size_t)j * 2 + 0) * L + i) * N + (size_t)tid * NQ::R;
-                        const size_t oa = (((size_t)j * 2 + 1) * L + i) * N + (size_t)tid * NQ::R;
+                        const ulonglong2* kb = key + (((size_t)j * 2 + 0) * L + i) * N;
+                        const ulonglong2* ka = key + (((size_t)j * 2 + 1) * L + i) * N;
 #pragma unroll
-                        for (int v = 0; v < NQ::R; v += 2) {
-                            const ulonglong2 wb = __ldg(reinterpret_cast<const ulonglong2*>(rlk + ob + v));
-                            const ulonglong2 sb = __ldg(reinterpret_cast<const ulonglong2*>(rlk_sh + ob + v));
-                            const ulonglong2 wa = __ldg(reinterpret_cast<const ulonglong2*>(rlk + oa + v));
-                            const ulonglong2 sa = __ldg(reinterpret_cast<const ulonglong2*>(rlk_sh + oa + v));
-                            cs[cpos(v)] += shoup_lazy(x[v], wb.x, sb.x, m.q);
-                            cs[cpos(v + 1)] += shoup_lazy(x[v + 1], wb.y, sb.y, m.q);
-                            cs[N + cpos(v)] += shoup_lazy(x[v], wa.x, sa.x, m.q);
-                            cs[N + cpos(v + 1)] += shoup_lazy(x[v + 1], wa.y, sa.y, m.q);
+                        for (int v = 0; v < NQ::R; v++) {
+                            const int e = NQ::lane_idx(v, tid);
+                            const ulonglong2 wb = __ldg(kb + e), wa = __ldg(ka + e);
+                            cs[e] += (u64)pm_mul((i64)x[v], wb.x, wb.y, pc);
+                            cs[N + e] += (u64)pm_mul((i64)x[v], wa.x, wa.y, pc);
                         }
                     }
                 }
-                u64* c0 = Cout + (size_t)i * N + (size_t)tid * NQ::R;
-                u64* c1 = Cout + ((size_t)L + i) * N + (size_t)tid * NQ::R;
+                for (int p = 0; p < 2; p++) {
+                    u64 x[NQ::R];
 #pragma unroll
-                for (int v = 0; v < NQ::R; v += 2) {
-                    *reinterpret_cast<ulonglong2*>(c0 + v) =
-                        make_ulonglong2(barrett64(cs[cpos(v)], m), barrett64(cs[cpos(v + 1)], m));
-                    *reinterpret_cast<ulonglong2*>(c1 + v) =
-                        make_ulonglong2(barrett64(cs[N + cpos(v)], m), barrett64(cs[N + cpos(v + 1)], m));
+                    for (int v = 0; v < NQ::R; v++) x[v] = cs[(size_t)p * N + NQ::lane_idx(v, tid)];
+                    NQ::run_to_lane(x, sm, tid);
+                    u64* dst = Cout + ((size_t)p * L + i) * N;
+#pragma unroll
+                    for (int v = 0; v < NQ::R; v++) dst[NQ::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
                 }
             }
         } else {
             // the L + 2 forward transforms of a limb run with 16 words per
             // thread (two virtual threads of the 16-word geometry per thread,
             // the data in shared memory between passes), which keeps stage R
-            // within the registers the CTA is launched with
-            using NH = NttT<LOGN, 4, Arith64>;
-            constexpr int VT = NH::NT / NTH;
-            static_assert(NH::SMEM_WORDS * 8 <= PP::SMEM, "shared memory of the looped transform");
-            u64* U = reinterpret_cast<u64*>(T);  // [L + 2][N], slot e at its place
+            // within the registers the CTA is launched with; U and the sums
+            // stay lane-interleaved until the output
+            static_assert(NQ::SMEM_WORDS * 8 <= PP::SMEM, "shared memory of the looped transform");
+            u64* U = reinterpret_cast<u64*>(T);  // [L + 2][N], lane-interleaved
             for (int i = 0; i < L; i++) {
                 const Mod m = c.m[i];
+                const int pc = pm_c(m.q);
                 const u64* tw = c.tw + (size_t)i * 4 * N;
                 for (int s = 0; s < L + 2; s++) {
                     const u64* src = s < 2 ? acc + ((size_t)s * L + i) * N : acc + ((size_t)2 * L + (s - 2)) * N;
                     u64* dst = U + (size_t)s * N;
-                    NH::template forward_looped<VT>(
-                        sm, tid, tw, m.q, [&](int e) { return barrett64(src[e], m); },
-                        [&](int vt, const u64(&x)[NH::R]) {
+                    NQ::template forward_looped<VT>(
+                        sm, tid, tw, m.q, [&](int e) { return (u64)pm_fold_u(src[e], pc); },
+                        [&](int vt, const u64(&x)[NQ::R]) {
 #pragma unroll
-                            for (int v = 0; v < NH::R; v += 2)
-                                *reinterpret_cast<ulonglong2*>(dst + (size_t)vt * NH::R + v) = make_ulonglong2(x[v], x[v + 1]);
+                            for (int v = 0; v < NQ::R; v++) dst[NQ::lane_idx(v, vt)] = x[v];
                         });
                 }
-                // every thread reads back the slots its virtual threads wrote
+                // every thread reads back the words its virtual threads wrote
+                for (int p = 0; p < 2; p++) {
+                    __syncthreads();  // the shared memory is free
 #pragma unroll 1
-                for (int jv = 0; jv < VT; jv++) {
-                const size_t e0 = (size_t)(tid + jv * NTH) * NH::R;
-                u64* c0 = Cout + (size_t)i * N + e0;
-                u64* c1 = Cout + ((size_t)L + i) * N + e0;
-#pragma unroll 1
-                for (int v = 0; v < NH::R; v += 2) {
-                    const ulonglong2 u0 = *reinterpret_cast<const ulonglong2*>(U + e0 + v);
-                    const ulonglong2 u1 = *reinterpret_cast<const ulonglong2*>(U + N + e0 + v);
-                    u64 b0 = u0.x, b1 = u0.y, a0 = u1.x, a1 = u1.y;
+                    for (int vt = tid; vt < NQ::NT; vt += NTH) {
+#pragma unroll 2
+                        for (int v = 0; v < NQ::R; v++) {
+                            const int e = NQ::lane_idx(v, vt);
+                            i64 t = (i64)U[(size_t)p * N + e];
 #pragma unroll
-                    for (int j = 0; j < L; j++) {
-                        const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(U + (size_t)(2 + j) * N + e0 + v);
-                        const size_t ob = (((size_t)j * 2 + 0) * L + i) * N + e0 + v;
-                        const size_t oa = (((size_t)j * 2 + 1) * L + i) * N + e0 + v;
-                        const ulonglong2 wb = __ldg(reinterpret_cast<const ulonglong2*>(rlk + ob));
-                        const ulonglong2 sb = __ldg(reinterpret_cast<const ulonglong2*>(rlk_sh + ob));
-                        const ulonglong2 wa = __ldg(reinterpret_cast<const ulonglong2*>(rlk + oa));
-                        const ulonglong2 sa = __ldg(reinterpret_cast<const ulonglong2*>(rlk_sh + oa));
-                        b0 += shoup_lazy(d.x, wb.x, sb.x, m.q);
-                        b1 += shoup_lazy(d.y, wb.y, sb.y, m.q);
-                        a0 += shoup_lazy(d.x, wa.x, sa.x, m.q);
-                        a1 += shoup_lazy(d.y, wa.y, sa.y, m.q);
+                            for (int j = 0; j < L; j++) {
+                                const ulonglong2 w = __ldg(key + (((size_t)j * 2 + p) * L + i) * N + e);
+                                t += pm_mul((i64)U[(size_t)(2 + j) * N + e], w.x, w.y, pc);
+                            }
+                            sm[NQ::pad(NQ::run_idx(v, vt))] = pm_canon(t, m.q);
+                        }
                     }
-                    *reinterpret_cast<ulonglong2*>(c0 + v) = make_ulonglong2(barrett64(b0, m), barrett64(b1, m));
-                    *reinterpret_cast<ulonglong2*>(c1 + v) = make_ulonglong2(barrett64(a0, m), barrett64(a1, m));
-                }
+                    __syncthreads();
+                    u64* dst = Cout + ((size_t)p * L + i) * N;
+#pragma unroll 4
+                    for (int e = tid; e < N; e += NTH) dst[e] = sm[NQ::pad(e)];
                 }
             }
         }

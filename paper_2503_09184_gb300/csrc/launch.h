@@ -24,7 +24,7 @@ int ext_interleave(int logN);
 cudaError_t launch_ntt32(const RnsConsts& rc, bool inverse, const u32* in, size_t in_gstride, int in_l0, u32* out,
                          size_t out_gstride, int out_l0, int prime0, int nlimbs, long long ngroups, bool interleaved,
                          cudaStream_t s);
-cudaError_t launch_keygen(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_sh, int* err,
+cudaError_t launch_keygen(const RnsConsts& rc, u64* s_ntt, signed char* s_coeff, u64* rlk, u64* rlk_pm, int* err,
                           cudaStream_t s);
 cudaError_t launch_encrypt(const RnsConsts& rc, const u64* s_ntt, const long long* vals, const int* coords, long long n,
                            u64 matrix_id, u64* ct, int* err, cudaStream_t s);
@@ -35,19 +35,17 @@ cudaError_t launch_lift_extend(const RnsConsts& rc, const u64* in, u32* out, lon
 cudaError_t launch_tensor_intt(const RnsConsts& rc, const u32* a, const u32* b, u32* T, cudaStream_t s);
 cudaError_t launch_scale_round(const RnsConsts& rc, const u32* T, u64* D, cudaStream_t s);
 cudaError_t launch_relin_ntt(const RnsConsts& rc, const u64* D, u64* U, cudaStream_t s);
-cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk, const u64* rlk_sh, u64* C,
-                               cudaStream_t s);
+cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, cudaStream_t s);
 // fused persistent path (persistent_<logN>.cu).  One launch: the work list,
 // the key, the per-CTA scratch, the grid, the mode, the tile variant and a
-// persisting-L2 access-policy window (over the relinearisation key and its
-// companions; l2_bytes = 0: none).
+// persisting-L2 access-policy window (over the relinearisation key;
+// l2_bytes = 0: none).
 struct PersistentArgs {
     const MmDesc* mms;
     const Entry* entries;
     int n_entries;
     const int2* rowlist;
-    const u64* rlk;
-    const u64* rlk_sh;
+    const u64* rlk;  // in pm_mul's form: all w's, then all w2's
     u64* scratch;
     size_t scratch_stride;
     unsigned* queue;

@@ -22,9 +22,13 @@
 // forward's last pass is the same layout (stores are contiguous runs).
 //
 // Arithmetic policies (Harvey's lazy butterflies):
-//   Arith64, primes 2^53 < q < 2^54 in 64-bit words: forward accepts any
+//   Arith64, primes below 2^54 in 64-bit words: forward accepts any
 //     input below 2^63 and adds less than 2q per stage (no reductions);
 //     inverse keeps [0, 2q).
+//   Arith54, primes q = 2^54 - c in signed 64-bit words (pm_mul): forward
+//     accepts |x| < 2^58 and adds less than 2^55 per stage (no reductions);
+//     inverse doubles the sums' range at every stage and folds them once per
+//     FOLD_STAGES stages; outputs are reduced by canon().
 //   Arith32, primes 2^29 < b < 2^30 in 32-bit words: forward keeps [0, 4b)
 //     (input below 4b), inverse keeps [0, 2b).
 #pragma once
@@ -32,6 +36,8 @@
 
 struct Arith64 {
     using W = u64;
+    static constexpr int FOLD_STAGES = 0;
+    static constexpr bool PAIRS = false;
     template <bool LEAN>
     SFHE_DEV static void fwd(W& X, W& Y, W w, W ws, W q)
     {
@@ -55,8 +61,41 @@ struct Arith64 {
     }
 };
 
+struct Arith54 {
+    using W = u64;
+    // inverse: canonical inputs are below 2^54; after s stages without a fold
+    // the sums are below 2^(54+s), the differences fed to pm_mul below
+    // 2^(54+s): eight stages stay within its range
+    static constexpr int FOLD_STAGES = 8;
+    static constexpr bool PAIRS = true;  // twiddle layout: see tw_pair
+    SFHE_DEV static W fold(W x, W q) { return (W)pm_fold((i64)x, pm_c(q)); }
+    SFHE_DEV static W canon(W x, W q) { return pm_canon((i64)x, q); }
+    template <bool LEAN>
+    SFHE_DEV static void fwd(W& X, W& Y, W w, W w2, W q)
+    {
+        const W T = (W)pm_mul((i64)Y, w, w2, pm_c(q));
+        Y = X - T;
+        X = X + T;
+    }
+    template <bool LEAN>
+    SFHE_DEV static void inv(W& X, W& Y, W w, W w2, W q)
+    {
+        const W s = X + Y, d = X - Y;
+        X = s;
+        Y = (W)pm_mul((i64)d, w, w2, pm_c(q));
+    }
+    SFHE_DEV static void inv_last(W& X, W& Y, W ni, W ni2, W wl, W wl2, W q)
+    {
+        const W s = X + Y, d = X - Y;
+        X = (W)pm_mul((i64)s, ni, ni2, pm_c(q));
+        Y = (W)pm_mul((i64)d, wl, wl2, pm_c(q));
+    }
+};
+
 struct Arith32 {
     using W = u32;
+    static constexpr int FOLD_STAGES = 0;
+    static constexpr bool PAIRS = false;
     // LEAN: min(s, s - 2b) reduces s < 4b to [0, 2b) (below 2b the
     // difference wraps above 2^31 > s); otherwise a compare and select
     SFHE_DEV static W red2(W s, W b) { return s >= 2 * b ? s - 2 * b : s; }
@@ -177,6 +216,29 @@ struct NttT {
         for (int v = 0; v < R; v++) x[v] = sm[LEAN ? slot_addr<S, RR>(base, v) : pad(idx<S, RR>(v, tid))];
     }
 
+    // Between the run layout and the coalesced one (slot v of thread tid:
+    // element v NT + tid), one exchange: NTT-form words in natural order are
+    // read and written by consecutive lanes at consecutive addresses (a warp's
+    // 64-bit accesses in the run layout touch 32 separate 128-byte lines).
+    SFHE_DEV static void run_to_lane(W (&x)[R], W* sm, int tid)
+    {
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < R; v++) sm[pad(run_idx(v, tid))] = x[v];
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < R; v++) x[v] = sm[pad(lane_idx(v, tid))];
+    }
+    SFHE_DEV static void lane_to_run(W (&x)[R], W* sm, int tid)
+    {
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < R; v++) sm[pad(lane_idx(v, tid))] = x[v];
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < R; v++) x[v] = sm[pad(run_idx(v, tid))];
+    }
+
     // The C twiddles (and Shoup companions) at w[ti0 .. ti0+C-1]; ti0 is a
     // multiple of C, so they come in as 16-byte (or 8-byte) vector loads.
     template <int C>
@@ -206,6 +268,22 @@ struct NttT {
             }
         }
     }
+    // Arith54's tables hold the two words of a twiddle side by side (one
+    // 16-byte load), and the levels of the pass at S = 0, where thread G uses
+    // C = base / NT consecutive twiddles of the level starting at `base`, are
+    // stored lane-interleaved (twiddle t of thread G at base + t NT + G), so
+    // that a warp reads consecutive bytes instead of one 64-byte run per lane.
+    template <int S, int CB>
+    SFHE_DEV static void tw_pair(W (&wv)[CB], W (&wsv)[CB], const W* __restrict__ w, int base, int C, int G, int t0)
+    {
+#pragma unroll
+        for (int t = 0; t < CB; t++) {
+            const int i = S == 0 ? base + (t0 + t) * NT + G : base + (G >> S) * C + t0 + t;
+            const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(w) + i);
+            wv[t] = p.x;
+            wsv[t] = p.y;
+        }
+    }
     // twiddles held in registers at a time: 64 bytes of each table (32 when
     // a thread holds 32 elements)
     static constexpr int TWB = (R >= 32 ? 32 : 64) / (int)sizeof(W);
@@ -230,7 +308,8 @@ struct NttT {
 #pragma unroll
                 for (int t0 = 0; t0 < C; t0 += CB) {
                     W wv[CB], wsv[CB];
-                    tw_fetch<CB>(wv, wsv, w, ws, ti0 + t0);
+                    if constexpr (A::PAIRS) tw_pair<S, CB>(wv, wsv, w, 1 << lvl, C, G, t0);
+                    else tw_fetch<CB>(wv, wsv, w, ws, ti0 + t0);
 #pragma unroll
                     for (int t = 0; t < CB; t++) {
 #pragma unroll
@@ -286,7 +365,7 @@ struct NttT {
     // stores them back in place, so only R elements are live per thread at a
     // time (the register-resident forward above keeps all of a thread's
     // elements across the passes).  in(e) returns input element e (natural
-    // order, below 2^63); out(vt, x) receives the R outputs of virtual
+    // order, within the policy's input range); out(vt, x) receives the R outputs of virtual
     // thread vt, slots vt R .. vt R + R - 1 (the run layout).  sm holds
     // SMEM_WORDS words.
     template <int VT, typename In, typename Out>
@@ -358,7 +437,10 @@ struct NttT {
 #pragma unroll
                 for (int t0 = 0; t0 < C; t0 += CB) {
                     W wv[CB], wsv[CB];
-                    if constexpr (!(LAST && D == RR - 1)) tw_fetch<CB>(wv, wsv, w, ws, ti0 + t0);
+                    if constexpr (!(LAST && D == RR - 1)) {
+                        if constexpr (A::PAIRS) tw_pair<S, CB>(wv, wsv, w, N >> (S + D + 1), C, G, t0);
+                        else tw_fetch<CB>(wv, wsv, w, ws, ti0 + t0);
+                    }
 #pragma unroll
                     for (int t = 0; t < CB; t++) {
 #pragma unroll
@@ -391,10 +473,34 @@ struct NttT {
         for (int j = 0; j < NP; j++) load<S1, RR1>(x[j], sm + (size_t)j * SMEM_WORDS, tid);
     }
 
+    // Arith54: fold every sum before pass PS when the stages since the last
+    // fold and those of the pass would exceed FOLD_STAGES
+    static constexpr __host__ __device__ int pass_stages(int ps) { return ps < NFULL ? LOGR : REM; }
+    static constexpr __host__ __device__ int stages_since_fold(int ps)  // before pass ps, its own fold not counted
+    {
+        int s = 0;
+        for (int p = 0; p < ps; p++) s = (s + pass_stages(p) > A::FOLD_STAGES ? 0 : s) + pass_stages(p);
+        return s;
+    }
+    template <int NP, int PS>
+    SFHE_DEV static void fold_before(W (&x)[NP][R], W q)
+    {
+        if constexpr (A::FOLD_STAGES > 0) {
+            if constexpr (stages_since_fold(PS) + pass_stages(PS) > A::FOLD_STAGES) {
+#pragma unroll
+                for (int j = 0; j < NP; j++) {
+#pragma unroll
+                    for (int v = 0; v < R; v++) x[j][v] = A::fold(x[j][v], q);
+                }
+            }
+        }
+    }
+
     template <int NP, int PS>
     SFHE_DEV static void inv_rest(W (&x)[NP][R], W* sm, int tid, const W* w, const W* ws, W q, W ni, W nis, W wl,
                                   W wls)
     {
+        fold_before<NP, PS>(x, q);
         if constexpr (PS < NFULL) {
             exchange<NP, (PS - 1) * LOGR, LOGR, PS * LOGR, LOGR>(x, sm, tid);
             inv_stages<NP, PS * LOGR, LOGR, (PS == NFULL - 1 && REM == 0), 0>(x, tid, w, ws, q, ni, nis, wl, wls);
@@ -490,11 +596,6 @@ struct NttT {
 // base) transforms; R elements per thread, N / R threads per CTA.
 template <int LOGN>
 struct NttGeom {
-    using T = NttT<LOGN, 4, Arith64>;
-    using T32 = NttT<LOGN, 4, Arith32>;
-};
-template <>
-struct NttGeom<14> {
-    using T = NttT<14, 5, Arith64>;
-    using T32 = NttT<14, 5, Arith32>;
+    using T = NttT<LOGN, 4, Arith54>;
+    using T32 = NttT<LOGN, LOGN == 14 ? 5 : 4, Arith32>;
 };

@@ -23,7 +23,7 @@ static int occupancy_of()
     int blocks = 0;
     const size_t smem = PersistentPlan<LOGN, L>::SMEM;
     if (allow_smem(k_matmul_persistent<LOGN, L, false, 0>, smem) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_matmul_persistent<LOGN, L, false, 0>, nt_of<LOGN>(),
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_matmul_persistent<LOGN, L, false, 0>, NttGeom<LOGN>::T32::NT,
                                                       smem) != cudaSuccess)
         return 0;
     return blocks;
@@ -52,7 +52,7 @@ static cudaError_t launch_instance(const RnsConsts& rc, const PersistentArgs& a,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.grid);
-    cfg.blockDim = dim3((unsigned)nt_of<LOGN>());
+    cfg.blockDim = dim3((unsigned)NttGeom<LOGN>::T32::NT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -66,7 +66,7 @@ static cudaError_t launch_instance(const RnsConsts& rc, const PersistentArgs& a,
         cfg.attrs = attr;
         cfg.numAttrs = 1;
     }
-    return cudaLaunchKernelEx(&cfg, kern, rc, a.mms, a.entries, a.n_entries, a.rowlist, a.rlk, a.rlk_sh, a.scratch,
+    return cudaLaunchKernelEx(&cfg, kern, rc, a.mms, a.entries, a.n_entries, a.rowlist, a.rlk, a.scratch,
                               a.scratch_stride, a.queue, a.stop);
 }
 

@@ -35,6 +35,14 @@ struct ShoupC {
     u64 ws;
 };
 
+// A constant multiplier w modulo q = 2^54 - c, prepared for pm_mul: w and
+// 2^32 w mod q, each centred (|.| <= q / 2) and packed as its floor quotient
+// by 2^22 (signed, high word) and its remainder (22 bits, low word).
+struct PmC {
+    u64 w;
+    u64 w2;
+};
+
 // A 30-bit modulus b with floor(2^61 / b) (values below 2^61) and
 // floor(2^64 / b) (any 64-bit value).
 struct Mod32 {
@@ -59,11 +67,13 @@ struct RnsConsts {
     Mod m[SFHE_MAX_L];
     Mod32 mb[SFHE_MAX_K];
     // NTT twiddles in device memory: Q primes [L][4][N] u64, B primes
-    // [K][4][N] u32; rows psi_rev, psi_rev_shoup, ipsi_rev, ipsi_rev_shoup
-    // (psi^(+-bitrev(k)), psi the smallest primitive 2N-th root).
+    // [K][4][N] u32 (psi^(+-bitrev(k)), psi the smallest primitive 2N-th
+    // root): over Q pairs PmC of psi_rev, then of ipsi_rev (twiddles_pm's
+    // order); over B rows psi_rev, psi_rev_shoup, ipsi_rev, ipsi_rev_shoup.
     const u64* tw;
     const u32* twb;
-    ShoupC ninv[SFHE_MAX_L], wlast[SFHE_MAX_L];
+    ShoupC ninv[SFHE_MAX_L];
+    PmC ninv_pm[SFHE_MAX_L], wlast_pm[SFHE_MAX_L];
     Shoup32 ninv_b[SFHE_MAX_K], wlast_b[SFHE_MAX_K];
     // the same multiplied by 2^32 (B/b_k)^-1: an inverse NTT of the tensor in
     // Montgomery form with these outputs x~_k = [x_k (B/b_k)^-1]_{b_k}

@@ -69,10 +69,12 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_galois_keygen(const __
     u64* bs_out = key_sh + (((size_t)j * 2 + 0) * L + i) * N;
     u64* as_out = key_sh + (((size_t)j * 2 + 1) * L + i) * N;
     const u64* s = s_ntt + (size_t)i * N;
+    NT_::run_to_lane(a, sm, tid);
+    NT_::run_to_lane(e, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
-        const int k = NT_::run_idx(v, tid);
-        const u64 av = barrett64(a[v], m), ev = barrett64(e[v], m);
+        const int k = NT_::lane_idx(v, tid);
+        const u64 av = pm_canon((i64)a[v], m.q), ev = pm_canon((i64)e[v], m.q);
         u64 bv = sub_mod(ev, mul_mod(av, s[k], m), m.q);
         if (i == j) bv = add_mod(bv, s[galois_src<LOGN>(k, g)], m.q);
         b_out[k] = bv;
@@ -116,11 +118,13 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_encrypt_poly(const __g
     NT_::forward(e, sm, tid, tw, m.q);
     u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
     u64* c1 = c0 + (size_t)L * N;
+    NT_::run_to_lane(a, sm, tid);
+    NT_::run_to_lane(e, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
-        const int k = NT_::run_idx(v, tid);
-        const u64 av = barrett64(a[v], m);
-        c0[k] = sub_mod(barrett64(e[v], m), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
+        const int k = NT_::lane_idx(v, tid);
+        const u64 av = pm_canon((i64)a[v], m.q);
+        c0[k] = sub_mod(pm_canon((i64)e[v], m.q), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
         c1[k] = av;
     }
     if (fail) atomicExch(err, 1);
@@ -254,8 +258,9 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_ks_ntt(const __grid_co
     for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::fwd_in_idx(v, tid)];
     NT_::forward(x, sm, tid, c.tw + (size_t)i * 4 * N, m.q);
     u64* dst = U + blockIdx.z * u_stride + ((size_t)s * L + i) * N;
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) dst[NT_::run_idx(v, tid)] = barrett64(x[v], m);
+    for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
 }
 
 // out[p][i] = U[p][i] + sum_j U[2+j][i] key[j][p][i]   (p = 0: b, 1: a)
@@ -469,10 +474,15 @@ cudaError_t launch_rotate(const RnsConsts& rc, const u64* in, u32 g, const u64* 
     if (e == cudaSuccess) e = launch_ntt(rc, true, P, LN, 0, D, LN, 0, 0, rc.L, 1, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(D + LN, 0, LN * 8, s);
     if (e == cudaSuccess) e = launch_ntt(rc, true, P + LN, LN, 0, D + 2 * LN, LN, 0, 0, rc.L, 1, s);
-    if (e == cudaSuccess) e = launch_relin_ntt(rc, D, U, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, 2 * LN * 8, s);
-    if (e == cudaSuccess) e = launch_relin_accum(rc, U, key, key_sh, out, s);
-    return e;
+    if (e != cudaSuccess) return e;
+    SLOTS_DISPATCH_LOGN(rc.logN, {
+        if ((e = allow_smem(k_ks_ntt<LG>, smem_of<LG>())) != cudaSuccess) return e;
+        k_ks_ntt<LG><<<dim3(rc.L, rc.L + 2, 1), nt_of<LG>(), smem_of<LG>(), s>>>(rc, D, 0, U, 0);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        break;
+    });
+    k_ks_accum<<<dim3((unsigned)((rc.N + 255) / 256), rc.L, 1), 256, 0, s>>>(rc, U, 0, key, key_sh, out, 0);
+    return cudaGetLastError();
 }
 
 }  // namespace sfhe
