@@ -5,7 +5,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <mutex>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -103,7 +105,10 @@ struct sfhe_plan {
     sfhe_ctx* ctx;
     uint32_t flags;
     std::vector<MmDesc> mms;
-    std::vector<Entry> entries;
+    std::vector<Entry> entries;   // units: whole output entries or parts of one
+    int64_t out_entries = 0;      // output entries
+    int slots = 0;                // partial-sum slots of the shared-out entries
+    std::vector<int> last_unit;   // with slots: per output entry its last unit, ascending
     std::vector<int2> rowlist;
     std::vector<size_t> c_words;  // per matmul: words of C
     int64_t products;
@@ -114,6 +119,9 @@ struct sfhe_plan {
     int2* d_rowlist;
     u64* d_scratch;
     size_t scratch_stride;
+    u64* d_partial;
+    unsigned* d_finished;
+    size_t queue_bytes;  // queue words and `finished`, cleared by every execution
     int grid;
     u32* d_T;
     u64 *d_D, *d_U;
@@ -543,7 +551,7 @@ extern "C" sfhe_status sfhe_export_relin_key(sfhe_ctx* c, uint64_t* out, void* s
 namespace {
 
 struct Layout {
-    size_t queue, mms, entries, rowlist, scratch, T, D, U, total;
+    size_t queue, mms, entries, rowlist, scratch, partial, T, D, U, total;
 };
 
 sfhe_status validate_matrix(const sfhe_matrix_view& m, const char* name)
@@ -680,13 +688,110 @@ sfhe_status build(const sfhe_ctx* c, int32_t n, const sfhe_matrix_view* A, const
     return SFHE_OK;
 }
 
+// Units of work of a persistent plan.  A CTA takes one unit at a time, so a
+// plan with few output entries (64 of the tiny workload on 304 resident CTAs)
+// leaves SMs idle, and one with a few times as many entries as CTAs ends on an
+// uneven last round.  Below 8 entries per CTA the products of an entry may
+// therefore be shared out over several units of at most u products; the last
+// unit to finish adds the sums up and relinearises.  u is the one whose
+// longest-first schedule is estimated shortest, in units of a product: an
+// entry's relinearisation counts 0.6 (N = 8192, L = 4: 1.17 us per entry
+// against 1.89 us per product, full chip) and a part 0.15 (its sums are
+// written and read once more).  In the grouped mode a unit holds whole rounding groups.
+// Measured (GB300): tiny 8^3 replay 502 -> 303 us, 13 x 29 x 7 one-shot 4.07 ->
+// 2.54 ms.  More than 2 units per CTA are not made (the slots' memory).
+const double kRelinCost = 0.6, kPartCost = 0.15;
+
+double schedule_length(const std::vector<double>& cost, int grid)
+{
+    // longest first onto the least loaded CTA
+    std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+    double end = 0;
+    for (double x : cost) {
+        double t = x;
+        if ((int)load.size() >= grid) {
+            t += load.top();
+            load.pop();
+        }
+        load.push(t);
+        end = std::max(end, t);
+    }
+    return end;
+}
+
+void split_entries(const sfhe_ctx* c, sfhe_plan& P, uint32_t flags)
+{
+    P.out_entries = (int64_t)P.entries.size();
+    P.slots = 0;
+    P.last_unit.clear();
+    for (Entry& e : P.entries) e.parts = 1, e.slot = e.first_slot = 0;
+    if (!(flags & SFHE_EXEC_PERSISTENT) || P.entries.empty()) return;
+    const int grid = persistent_ctas_per_sm(c->rc) * c->num_sms;
+    const int granule = (flags & SFHE_EXEC_LAZY) ? c->rc.lazy_group : 1;
+    const int longest = P.entries[0].count;
+    if (grid <= 0 || P.out_entries >= 8 * (int64_t)grid || longest <= granule) return;
+    auto parts_of = [](int count, int u) { return count <= u ? 1 : (count + u - 1) / u; };
+    std::vector<double> cost;
+    double best = 0;
+    int best_u = 0, last_u = 0;
+    double work = 0;
+    for (const Entry& e : P.entries) work += e.count + kRelinCost;
+    // candidates in steps of about 4/3: this runs on the host in one-shot calls
+    for (int pieces = 1; pieces <= (longest + granule - 1) / granule && pieces <= 256; pieces += 1 + pieces / 3) {
+        const int u = (((longest + granule - 1) / granule + pieces - 1) / pieces) * granule;
+        if (u == last_u) continue;
+        last_u = u;
+        int64_t slots = 0;
+        cost.clear();
+        for (const Entry& e : P.entries) {
+            const int parts = parts_of(e.count, u);
+            if (parts > 1) slots += parts;
+            for (int p = 0; p < parts; p++)
+                cost.push_back(std::min(u, e.count - p * u) + (p == parts - 1 ? kRelinCost : 0.0) +
+                               (parts > 1 ? kPartCost : 0.0) + (p == parts - 1 && parts > 1 ? kPartCost * parts : 0.0));
+        }
+        if (slots > 2 * (int64_t)grid) break;
+        std::sort(cost.begin(), cost.end(), std::greater<double>());
+        const double t = schedule_length(cost, grid);
+        if (pieces == 1 || t < 0.97 * best) best = t, best_u = u;
+        if (best < 1.05 * work / grid) break;  // the chip is filled evenly
+    }
+    if (best_u >= longest) return;
+    std::vector<Entry> units;
+    for (const Entry& e : P.entries) {
+        const int parts = parts_of(e.count, best_u), first_slot = P.slots;
+        for (int p = 0; p < parts; p++) {
+            Entry x = e;
+            x.first = e.first + p * best_u;
+            x.count = std::min(best_u, e.count - p * best_u);
+            x.parts = parts;
+            x.first_slot = parts > 1 ? first_slot : 0;
+            x.slot = parts > 1 ? first_slot + p : 0;
+            units.push_back(x);
+        }
+        if (parts > 1) P.slots += parts;
+    }
+    std::stable_sort(units.begin(), units.end(), [](const Entry& a, const Entry& b) { return a.count > b.count; });
+    std::vector<int> last(P.slots, 0);  // by first slot
+    for (size_t i = 0; i < units.size(); i++) {
+        if (units[i].parts > 1) last[units[i].first_slot] = (int)i;
+        else P.last_unit.push_back((int)i);
+    }
+    for (const Entry& x : units)
+        if (x.parts > 1 && x.slot == x.first_slot) P.last_unit.push_back(last[x.first_slot]);
+    std::sort(P.last_unit.begin(), P.last_unit.end());
+    P.entries = std::move(units);
+}
+
+size_t partial_words(const RnsConsts& rc) { return (size_t)3 * rc.L * rc.N; }
+
 Layout layout_of(const sfhe_ctx* c, const sfhe_plan& P, uint32_t flags, int* grid_out, size_t* stride_out)
 {
     Layout Lo;
     memset(&Lo, 0, sizeof(Lo));
     size_t off = 0;
     Lo.queue = off;
-    off += 256;
+    off += 256 + align256((size_t)P.slots * sizeof(unsigned));  // `finished` behind the queue words
     Lo.mms = off;
     off += align256(P.mms.size() * sizeof(MmDesc));
     Lo.entries = off;
@@ -703,6 +808,8 @@ Layout layout_of(const sfhe_ctx* c, const sfhe_plan& P, uint32_t flags, int* gri
         const size_t stride = persistent_scratch_words(c->rc);
         Lo.scratch = off;
         off += align256((size_t)grid * stride * 8);
+        Lo.partial = off;
+        off += (size_t)P.slots * partial_words(c->rc) * 8;
         *grid_out = grid;
         *stride_out = stride;
     }
@@ -742,6 +849,8 @@ PersistentArgs persistent_args(const sfhe_plan* P, int n_entries, int variant)
     a.scratch_stride = P->scratch_stride;
     a.queue = P->d_queue;
     a.stop = P->d_stop;
+    a.partial = P->d_partial;
+    a.finished = P->d_finished;
     a.grid = P->grid;
     a.grouped = (P->flags & SFHE_EXEC_LAZY) != 0;
     a.variant = a.grouped ? 0 : variant;
@@ -764,7 +873,7 @@ sfhe_status tune_variants(sfhe_plan* P, cudaStream_t s)
     sfhe_ctx* c = P->ctx;
     const int nv = c->n_variants;
     std::vector<Entry> cal(P->entries.begin(), P->entries.begin() + std::min<size_t>(P->entries.size(), P->grid));
-    for (Entry& e : cal) e.count = std::min(e.count, 4);
+    for (Entry& e : cal) e.count = std::min(e.count, 4), e.parts = 1;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
@@ -810,7 +919,7 @@ sfhe_status launch_plan(sfhe_plan* P, cudaStream_t s)
             CUDA_TRY(cudaGraphLaunch(P->gexec, s));
             return SFHE_OK;
         }
-        CUDA_TRY(cudaMemsetAsync(P->d_queue, 0, 2 * sizeof(unsigned), s));
+        CUDA_TRY(cudaMemsetAsync(P->d_queue, 0, P->queue_bytes, s));
         if (P->entries.empty()) return SFHE_OK;
         CUDA_TRY(launch_persistent(rc, persistent_args(P, (int)P->entries.size(), P->variant), s));
         return SFHE_OK;
@@ -860,6 +969,10 @@ static sfhe_plan* new_plan(sfhe_ctx* c, uint32_t flags)
     P->gexec = nullptr;
     P->d_stop = nullptr;
     P->launched = false;
+    P->out_entries = 0;
+    P->slots = 0;
+    P->d_partial = nullptr;
+    P->d_finished = nullptr;
     return P;
 }
 
@@ -878,6 +991,7 @@ static sfhe_status plan_create_impl(sfhe_ctx* c, int32_t n, const sfhe_matrix_vi
         delete P;
         return st;
     }
+    split_entries(c, *P, flags);
     return plan_finish(c, P, flags, work, work_bytes, stream, out);
 }
 
@@ -901,6 +1015,9 @@ static sfhe_status plan_finish(sfhe_ctx* c, sfhe_plan* P, uint32_t flags, void* 
     P->d_entries = (Entry*)(w + Lo.entries);
     P->d_rowlist = (int2*)(w + Lo.rowlist);
     P->d_scratch = (u64*)(w + Lo.scratch);
+    P->d_partial = (u64*)(w + Lo.partial);
+    P->d_finished = (unsigned*)(w + Lo.queue + 256);
+    P->queue_bytes = P->slots ? 256 + (size_t)P->slots * sizeof(unsigned) : 2 * sizeof(unsigned);
     P->d_T = (u32*)(w + Lo.T);
     P->d_D = (u64*)(w + Lo.D);
     P->d_U = (u64*)(w + Lo.U);
@@ -938,7 +1055,7 @@ static sfhe_status plan_finish(sfhe_ctx* c, sfhe_plan* P, uint32_t flags, void* 
         if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             sfhe_status ls = SFHE_OK;
-            if (cudaMemsetAsync(P->d_queue, 0, 2 * sizeof(unsigned), cap) != cudaSuccess) ls = SFHE_ECUDA;
+            if (cudaMemsetAsync(P->d_queue, 0, P->queue_bytes, cap) != cudaSuccess) ls = SFHE_ECUDA;
             if (ls == SFHE_OK && !P->entries.empty())
                 if (launch_persistent(c->rc, persistent_args(P, (int)P->entries.size(), P->variant), cap) !=
                     cudaSuccess)
@@ -994,7 +1111,9 @@ extern "C" sfhe_status sfhe_plan_progress(const sfhe_plan* P, int64_t* done, voi
     CUDA_TRY(cudaStreamSynchronize(as_stream(stream)));
     unsigned taken = 0;
     CUDA_TRY(cudaMemcpy(&taken, P->d_queue, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    *done = std::min<int64_t>((int64_t)taken, (int64_t)P->entries.size());
+    // every unit taken by a launch that has ended is complete
+    const int64_t units = std::min<int64_t>((int64_t)taken, (int64_t)P->entries.size());
+    *done = P->slots ? std::lower_bound(P->last_unit.begin(), P->last_unit.end(), (int)units) - P->last_unit.begin() : units;
     return SFHE_OK;
 }
 
@@ -1044,7 +1163,7 @@ extern "C" sfhe_status sfhe_plan_stats(const sfhe_plan* P, int64_t* products, in
 {
     if (!P) return fail(SFHE_EINVAL, "null plan");
     if (products) *products = P->products;
-    if (entries) *entries = (int64_t)P->entries.size();
+    if (entries) *entries = P->out_entries;
     if (launches) *launches = (P->flags & SFHE_EXEC_PERSISTENT) ? (P->entries.empty() ? 0 : 1) : 4 * P->products;
     if (ctas) *ctas = P->grid;
     return SFHE_OK;
@@ -1088,6 +1207,7 @@ static sfhe_status size_impl(const sfhe_ctx* c, int32_t n, const sfhe_matrix_vie
     P.flags = flags;
     st = build(c, n, A, B, nullptr, dense_loop, P);
     if (st != SFHE_OK) return st;
+    split_entries(c, P, flags);
     int grid;
     size_t stride;
     *bytes = layout_of(c, P, flags, &grid, &stride).total;
@@ -1107,8 +1227,14 @@ extern "C" sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* c, int32_t ma
     off += align256((size_t)max_entries * sizeof(Entry));
     off += align256((size_t)max_products * sizeof(int2));
     const size_t N = c->rc.N, L = c->rc.L, K = c->rc.K;
-    if (flags & SFHE_EXEC_PERSISTENT)
-        off += align256((size_t)persistent_ctas_per_sm(c->rc) * c->num_sms * persistent_scratch_words(c->rc) * 8);
+    if (flags & SFHE_EXEC_PERSISTENT) {
+        const size_t grid = (size_t)persistent_ctas_per_sm(c->rc) * c->num_sms;
+        off += align256(grid * persistent_scratch_words(c->rc) * 8);
+        // split_entries: at most 2 units per CTA share entries out, of at
+        // least one product each; more units than entries in the list
+        const size_t slots = std::min<size_t>(2 * grid, (size_t)max_products);
+        off += align256(slots * sizeof(unsigned)) + align256(slots * sizeof(Entry)) + slots * partial_words(c->rc) * 8;
+    }
     if (flags & SFHE_EXEC_PLAIN)
         off += align256(3 * K * N * 4) + align256(3 * L * N * 8) + align256((L + 2) * L * N * 8);
     *bytes = off;

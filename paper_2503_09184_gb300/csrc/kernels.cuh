@@ -701,12 +701,14 @@ struct PersistentTile {
 // folded to canonical every 256 products), cacc [2][N] uint64, T [3][K][N]
 // uint32 (x~_k, the inverse NTT's output).  queue[0] is the entry counter, queue[1] the error word (1: a
 // bulk copy did not complete within the wait bound).  mbarriers 0 and 1
-// track the operand pairs of stage T.
+// track the operand pairs of stage T.  `entries` lists units of work: whole
+// output entries, or (few entries, see split_entries in api.cu) parts of an
+// entry's products whose sums meet in `partial` / `finished`.
 template <int LOGN, int L, bool GROUPED, int V>
 __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
     const __grid_constant__ RnsConsts c, const MmDesc* __restrict__ mms, const Entry* __restrict__ entries, int n_entries,
     const int2* __restrict__ rowlist, const u64* __restrict__ rlk, u64* scratch,
-    size_t scratch_stride, unsigned* queue, const unsigned* stop)
+    size_t scratch_stride, unsigned* queue, const unsigned* stop, u64* partial, unsigned* finished)
 {
     using CF = Cfg<LOGN, L>;
     using NQ = typename CF::NQ;
@@ -722,8 +724,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
     __shared__ __align__(8) u64 mbar[2];
     const int tid = threadIdx.x;
     u64* base = scratch + (size_t)blockIdx.x * scratch_stride;
-    u64* acc = base;                                        // [3][L][N] u64
-    u64* cacc = acc + (size_t)3 * L * N;                    // [2][N] u64
+    u64* cacc = base + (size_t)3 * L * N;                   // [2][N] u64, behind the sums [3][L][N]
     u32* T = reinterpret_cast<u32*>(cacc + (size_t)2 * N);  // [3][K][N] u32
     const size_t ext_words = (size_t)2 * K * N;
     const size_t ct_words = (size_t)2 * L * N;
@@ -787,6 +788,8 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
             for (size_t w = tid; w < ct_words; w += NTH) Cout[w] = 0;
             continue;
         }
+        // the sums [3][L][N] of this unit's products
+        u64* acc = en.parts > 1 ? partial + (size_t)en.slot * 3 * L * N : base;
         auto operands = [&](int pr, const u32*& a, const u32*& b) {
             const int2 it = rowlist[en.first + pr];
             a = mm.A_ext + (size_t)it.x * ext_words;
@@ -1205,6 +1208,38 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                 __syncthreads();
             }
             }
+        }
+        // A unit of a shared-out entry leaves its sums in its slot; the unit
+        // that finishes last (no unit waits for another) adds the slots up and
+        // goes on to stage R.
+        if (en.parts > 1) {
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_entry = (int)atomicAdd(finished + en.first_slot, 1u);
+            __syncthreads();
+            if (s_entry != en.parts - 1) {
+                if constexpr (PP::STAGED || PP::STAGED2) fence_proxy_async();
+                continue;
+            }
+            __threadfence();
+            if (tid == 0) finished[en.first_slot] = 0;  // for the plan's next execution
+            const u64* p0 = partial + (size_t)en.first_slot * 3 * L * N;
+            for (int l = 0; l < 3 * L; l++) {
+                // sums of d0 and d1 use the whole word: folded before they are added
+                const bool lazy = l < 2 * L;
+                const int pc = pm_c(c.m[l % L].q);
+#pragma unroll 2
+                for (int e = tid; e < N; e += NTH) {
+                    u64 t = 0;
+                    for (int p = 0; p < en.parts; p++) {
+                        const u64 w = __ldcg(p0 + ((size_t)p * 3 * L + l) * N + e);
+                        t += lazy ? (u64)pm_fold_u(w, pc) : w;
+                    }
+                    base[(size_t)l * N + e] = t;
+                }
+            }
+            acc = base;
+            __syncthreads();
         }
         // stage R.  The forward NTT leaves slot tid * R + v of every polynomial
         // with thread tid, so the key products and the output are private to

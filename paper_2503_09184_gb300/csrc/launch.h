@@ -50,6 +50,8 @@ struct PersistentArgs {
     size_t scratch_stride;
     unsigned* queue;
     const unsigned* stop;  // nullable: once *stop != 0, no CTA takes another entry
+    u64* partial;          // sums of shared-out entries' units, 3 L N words a slot
+    unsigned* finished;    // per first slot: units finished (0 between executions)
     int grid;
     bool grouped;
     int variant;

@@ -67,7 +67,7 @@ static cudaError_t launch_instance(const RnsConsts& rc, const PersistentArgs& a,
         cfg.numAttrs = 1;
     }
     return cudaLaunchKernelEx(&cfg, kern, rc, a.mms, a.entries, a.n_entries, a.rowlist, a.rlk, a.scratch,
-                              a.scratch_stride, a.queue, a.stop);
+                              a.scratch_stride, a.queue, a.stop, a.partial, a.finished);
 }
 
 template <int LOGN, int L>

@@ -16,5 +16,11 @@ struct Entry {
     int col;    // j
     int count;  // products
     int first;  // first (a_idx, k) pair in the row list
-    int pad[3];
+    // An output entry whose products are shared out over several units: their
+    // number, this unit's slot of partial sums and the entry's first slot
+    // (slots first_slot .. first_slot + parts - 1, and the counter of its
+    // finished units).  parts = 1: the whole entry.
+    int parts;
+    int slot;
+    int first_slot;
 };
