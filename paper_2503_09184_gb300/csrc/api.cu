@@ -109,6 +109,7 @@ struct sfhe_plan {
     int64_t out_entries = 0;      // output entries
     int slots = 0;                // partial-sum slots of the shared-out entries
     std::vector<int> last_unit;   // with slots: per output entry its last unit, ascending
+    std::vector<Entry> whole;     // with slots: the entries before they were shared out
     std::vector<int2> rowlist;
     std::vector<size_t> c_words;  // per matmul: words of C
     int64_t products;
@@ -780,7 +781,18 @@ void split_entries(const sfhe_ctx* c, sfhe_plan& P, uint32_t flags)
     for (const Entry& x : units)
         if (x.parts > 1 && x.slot == x.first_slot) P.last_unit.push_back(last[x.first_slot]);
     std::sort(P.last_unit.begin(), P.last_unit.end());
+    P.whole = std::move(P.entries);
     P.entries = std::move(units);
+}
+
+// back to whole entries
+void unsplit_entries(sfhe_plan& P)
+{
+    if (P.slots == 0) return;
+    P.entries = std::move(P.whole);
+    P.whole.clear();
+    P.last_unit.clear();
+    P.slots = 0;
 }
 
 size_t partial_words(const RnsConsts& rc) { return (size_t)3 * rc.L * rc.N; }
@@ -1004,6 +1016,13 @@ static sfhe_status plan_finish(sfhe_ctx* c, sfhe_plan* P, uint32_t flags, void* 
     if ((flags & SFHE_EXEC_PERSISTENT) && P->grid <= 0) {
         delete P;
         return fail(SFHE_ECUDA, "persistent kernel cannot be resident on this device");
+    }
+    if (work && work_bytes < Lo.total && P->slots) {
+        // a workspace that was sized for another product set of the same
+        // shapes (the dense loop over masked operands, say) may hold whole
+        // entries only
+        unsplit_entries(*P);
+        Lo = layout_of(c, *P, flags, &P->grid, &P->scratch_stride);
     }
     if (!work || work_bytes < Lo.total) {
         delete P;
