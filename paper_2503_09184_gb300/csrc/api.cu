@@ -16,6 +16,7 @@
 #include "../../include/sfhe.h"
 #include "api_internal.h"
 #include "host_math.h"
+#include "round_shape.h"
 #include "launch.h"
 #include "chunk_launch.h"
 
@@ -85,6 +86,7 @@ struct sfhe_ctx {
     RnsConsts rc;
     u64* d_tw;
     u32* d_twb;
+    uint16_t* d_mm_b;  // right operand of the rounding's matrix product
     u64* d_s;
     signed char* d_s_coeff;
     u64* d_rlk;     // the key, followed in the same allocation by
@@ -212,6 +214,7 @@ extern "C" void sfhe_ctx_destroy(sfhe_ctx* c)
     forget_static_scratch(c->device);
     cudaFree(c->d_tw);
     cudaFree(c->d_twb);
+    cudaFree(c->d_mm_b);
     cudaFree(c->d_s);
     cudaFree(c->d_s_coeff);
     cudaFree(c->d_rlk);  // both forms share the allocation
@@ -263,18 +266,22 @@ extern "C" sfhe_status sfhe_ctx_create(const sfhe_params* params, uint64_t seed,
     for (int k = 0; k < rc.K; k++)
         twiddles32(rc.mb[k].b, N, twb.data() + (size_t)k * 4 * N, &rc.ninv_b[k], &rc.wlast_b[k]);
     fold_tensor_scaling(rc);
+    std::vector<uint16_t> mm_b(8, 0);
+    if (round_on_tensor_cores(rc.K)) round_mma_constants(rc, mm_b);
 
     const size_t rlk_words = (size_t)L * 2 * L * N;
     if (cudaMalloc(&c->d_tw, tw.size() * 8) != cudaSuccess || cudaMalloc(&c->d_twb, twb.size() * 4) != cudaSuccess ||
-        cudaMalloc(&c->d_s, (size_t)L * N * 8) != cudaSuccess ||
+        cudaMalloc(&c->d_mm_b, mm_b.size() * 2) != cudaSuccess || cudaMalloc(&c->d_s, (size_t)L * N * 8) != cudaSuccess ||
         cudaMalloc(&c->d_s_coeff, N) != cudaSuccess || cudaMalloc(&c->d_rlk, 3 * rlk_words * 8) != cudaSuccess ||
         cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess)
         return bail(fail(SFHE_ENOMEM, "device allocation of the context failed"));
     c->d_rlk_pm = c->d_rlk + rlk_words;
     rc.tw = c->d_tw;
     rc.twb = c->d_twb;
+    rc.mm_b = c->d_mm_b;
     if (cudaMemcpy(c->d_tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->d_twb, twb.data(), twb.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->d_mm_b, mm_b.data(), mm_b.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess)
         return bail(fail(SFHE_ECUDA, "table upload failed"));
     cudaError_t e = launch_keygen(rc, c->d_s, c->d_s_coeff, c->d_rlk, c->d_rlk_pm, c->d_err, 0);

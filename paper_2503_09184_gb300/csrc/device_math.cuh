@@ -339,6 +339,10 @@ SFHE_DEV void mbar_init(u64* bar, u32 count)
 }
 // make initialised mbarriers visible to the async proxy (before their first use)
 SFHE_DEV void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+SFHE_DEV void mbar_arrive(u64* bar)
+{
+    asm volatile("{\n\t.reg .b64 s;\n\tmbarrier.arrive.shared::cta.b64 s, [%0];\n\t}" ::"r"(smem_addr(bar)) : "memory");
+}
 // the calling thread arrives and announces `bytes` of incoming transactions
 SFHE_DEV void mbar_arrive_expect_tx(u64* bar, u32 bytes)
 {
@@ -371,17 +375,23 @@ SFHE_DEV u64 global_ns()
 // attempts have failed or max_ns nanoseconds have passed, whichever comes
 // first (an attempt may itself suspend the thread for a hardware-defined
 // time, so the time bound is the one that holds in real time)
+SFHE_DEV bool mbar_try(u64* bar, u32 parity)
+{
+    u32 done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
 SFHE_DEV bool mbar_wait(u64* bar, u32 parity, u32 max_tries, u64 max_ns)
 {
+    // the clock is read only once a first attempt has failed
+    if (mbar_try(bar, parity)) return true;
     const u64 t0 = global_ns();
-    for (u32 i = 0; i < max_tries; i++) {
-        u32 done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(smem_addr(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
+    for (u32 i = 1; i < max_tries; i++) {
+        if (mbar_try(bar, parity)) return true;
         if (global_ns() - t0 > max_ns) return false;
     }
     return false;

@@ -1,5 +1,6 @@
 // host_math.cpp -- number theory on the host for the RNS bases.
 #include "host_math.h"
+#include "round_shape.h"
 
 #include <utility>
 
@@ -531,6 +532,134 @@ void fold_tensor_scaling(RnsConsts& rc)
         const uint64_t b = rc.mb[k].b, h = mulm(rc.bhat_inv[k].w, (1ULL << 32) % b, b);
         rc.ninv_bx[k] = shoup32_of(mulm(rc.ninv_b[k].w, h, b), b);
         rc.wlast_bx[k] = shoup32_of(mulm(rc.wlast_b[k].w, h, b), b);
+    }
+}
+
+// fp16 bits of an integer, |v| <= 2048
+static uint16_t half_of(int v)
+{
+    if (v == 0) return 0;
+    const uint16_t sign = v < 0 ? 0x8000 : 0;
+    uint32_t a = (uint32_t)(v < 0 ? -v : v);
+    int e = 0;
+    while ((2u << e) <= a) ++e;
+    return (uint16_t)(sign | ((e + 15) << 10) | ((a << (10 - e)) & 0x3FF));
+}
+
+// v = sum_j d_j 512^j, six digits in [-256, 255] (the top one up to 256)
+static void signed_digits(int64_t v, int (&d)[6])
+{
+    for (int j = 0; j < 6; ++j) {
+        if (j == 5) {
+            d[j] = (int)v;
+            break;
+        }
+        int64_t lo = v & 511;
+        if (lo >= 256) lo -= 512;
+        d[j] = (int)lo;
+        v = (v - lo) / 512;
+    }
+}
+
+void round_mma_constants(RnsConsts& rc, std::vector<uint16_t>& b)
+{
+    const int L = rc.L, K = rc.K;
+    const RoundShape sh = round_shape(L, K);
+    b.assign((size_t)sh.kc * sh.nc, 0);
+    auto at = [&](int n, int k) -> uint16_t& {
+        return b[((size_t)(n / 8) * (sh.kc / 8) + k / 8) * 64 + (n % 8) * 8 + k % 8];
+    };
+    Big Q = big(1);
+    for (int i = 0; i < L; ++i) mul_small(Q, rc.m[i].q);
+    // C = A Q + R with |R| <= Q / 2: R centred (its sign), and round(R 2^54 / Q)
+    auto centre = [&](Big R, uint64_t* A, int64_t& rho) {
+        Big twice = R;
+        shl(twice, 1);
+        const bool neg = greater(twice, Q);
+        if (neg) {
+            Big t = Q;
+            sub(t, R);
+            R = t;
+            for (int i = 0; i < L; ++i) A[i] = (A[i] + 1) % rc.m[i].q;
+        }
+        uint64_t quo = 0;
+        for (int bit = 0; bit < 55; ++bit) {  // floor(R 2^55 / Q)
+            shl(R, 1);
+            quo <<= 1;
+            if (!greater(Q, R)) {
+                sub(R, Q);
+                quo |= 1;
+            }
+        }
+        rho = (int64_t)((quo + 1) >> 1);
+        if (neg) rho = -rho;
+    };
+    const u128 join = 1 + (1 << 9) + (1 << 18);
+    const uint64_t magic = (uint64_t)ROUND_MAGIC * (uint64_t)join;
+    const int bias = 128;  // the left operand's bytes are less 128
+    __int128 rho_sum = 0;
+    int64_t v_sum = 0;
+    uint64_t alpha_sum[SFHE_MAX_L] = {};
+    for (int k = 0; k < K; ++k) {
+        // byte 0: t (B/b_k) = A Q + R; the next byte's is 256 times it
+        Big c = big(rc.t), quo, R;
+        for (int j = 0; j < K; ++j)
+            if (j != k) mul_small(c, rc.mb[j].b);
+        divmod(c, Q, quo, R);
+        uint64_t A[SFHE_MAX_L];
+        for (int i = 0; i < L; ++i) A[i] = mod_small(quo, rc.m[i].q);
+        for (int a = 0; a < 4; ++a) {
+            uint64_t Ac[SFHE_MAX_L];
+            memcpy(Ac, A, sizeof(Ac));
+            int64_t rho;
+            centre(R, Ac, rho);
+            int d[6];
+            signed_digits(rho, d);
+            rho_sum += rho;
+            for (int j = 0; j < 6; ++j) at(1 + j, 4 * k + a) = half_of(d[j]);
+            for (int i = 0; i < L; ++i) {
+                const uint64_t q = rc.m[i].q;
+                signed_digits(Ac[i] > q / 2 ? (int64_t)Ac[i] - (int64_t)q : (int64_t)Ac[i], d);
+                alpha_sum[i] = (alpha_sum[i] + Ac[i]) % q;
+                for (int j = 0; j < 6; ++j) at(round_mma_col(i) + j, 4 * k + a) = half_of(d[j]);
+            }
+            for (int s = 0; s < 8; ++s) {  // times 256
+                shl(R, 1);
+                const uint64_t carry = greater(Q, R) ? 0 : 1;
+                if (carry) sub(R, Q);
+                for (int i = 0; i < L; ++i) A[i] = (2 * A[i] + carry) % rc.m[i].q;
+            }
+        }
+        const uint64_t bk = rc.mb[k].b;
+        const int c3 = (int)(((1ull << 40) + bk / 2) / bk), c2 = (int)(((1ull << 32) + bk / 2) / bk);
+        at(0, 4 * k + 3) = half_of(c3);
+        at(0, 4 * k + 2) = half_of(c2);
+        v_sum += c3 + c2;
+    }
+    rc.mm_p9 = 1u << 9, rc.mm_p18 = 1u << 18, rc.mm_p27 = 1u << 27;
+    rc.mm_vc = (uint32_t)(bias * v_sum + (1 << 15)) - ROUND_MAGIC;
+    for (int n = 0; n < sh.nc; ++n) at(n, 4 * K) = 0x6E00;  // 6144
+    // t B = alpha_B Q + r_B
+    Big cB = big(rc.t), quo, R;
+    for (int k = 0; k < K; ++k) mul_small(cB, rc.mb[k].b);
+    divmod(cB, Q, quo, R);
+    uint64_t AB[SFHE_MAX_L];
+    for (int i = 0; i < L; ++i) AB[i] = mod_small(quo, rc.m[i].q);
+    int64_t rhoB;
+    centre(R, AB, rhoB);
+    const int64_t nb = -rhoB, nb0 = nb & ((1 << 27) - 1);
+    rc.mm_rb0n = (int)nb0;
+    rc.mm_rb1n = (int)((nb - nb0) / (1 << 27));
+    const __int128 g = bias * rho_sum, gl = g & ((1 << 27) - 1);
+    rc.mm_g0 = (uint64_t)gl - magic;
+    rc.mm_g1 = (uint64_t)(int64_t)((g - gl) / (1 << 27)) + (1ull << 47) - magic;
+    for (int i = 0; i < L; ++i) {
+        const uint64_t q = rc.m[i].q, n = (q - AB[i]) % q;
+        rc.mm_nab_lo[i] = (uint32_t)(n & ((1 << 27) - 1));
+        rc.mm_nab_hi[i] = (uint32_t)(n >> 27);
+        // bias sum A - 2^20 - magic (1 + 2^27)
+        const uint64_t off = (uint64_t)(((u128)magic * ((1ull << 27) + 1) + (1 << 20)) % q);
+        rc.mm_cq[i] = (mulm(alpha_sum[i], (uint64_t)bias, q) + q - off) % q;
     }
 }
 

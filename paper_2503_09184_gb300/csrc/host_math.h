@@ -39,5 +39,8 @@ bool fill_constants(RnsConsts& rc);
 // (fill_constants): the tensor stage's inverse NTT takes its input in
 // Montgomery form and outputs x~_k.
 void fold_tensor_scaling(RnsConsts& rc);
+// The mm_ constants and the right operand of the rounding on the tensor
+// cores (round_mma.cuh), in the order its shared-memory copy has.
+void round_mma_constants(RnsConsts& rc, std::vector<uint16_t>& b);
 
 }  // namespace sfhe

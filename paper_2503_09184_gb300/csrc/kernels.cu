@@ -275,9 +275,8 @@ static_assert(PersistentTile<13, 4, 3>::SM == 2 && PersistentTile<13, 4, 3>::LS 
 static_assert(PersistentTile<13, 4, 4>::SM == 2 && PersistentTile<13, 4, 4>::LS == 2 &&
                   PersistentTile<13, 4, 4>::NB::SHUF, "tile table");
 static_assert(!PersistentTile<13, 4, 1>::NB::LEAN && !PersistentTile<13, 4, 1>::NB::SHUF, "tile table");
-static_assert(PersistentTile<14, 8, 0>::SM == 1 && PersistentTile<14, 8, 0>::LS == 8, "tile table");
-static_assert(PersistentTile<14, 8, 1>::SM == 1 && PersistentTile<14, 8, 1>::LS == 4, "tile table");
-static_assert(PersistentTile<14, 8, 2>::SM == 1 && PersistentTile<14, 8, 2>::LS == 2, "tile table");
+static_assert(PersistentTile<14, 8, 0>::MMA && !PersistentTile<14, 8, 0>::EARLY && PersistentTile<14, 8, 1>::EARLY &&
+                  PersistentTile<14, 8, 1>::NB::LEAN && !PersistentTile<14, 8, 2>::NB::LEAN, "tile table");
 static_assert(PersistentTile<12, 2, 0>::SM == 2 && PersistentTile<12, 2, 0>::LS == 2, "tile table");
 static_assert(PersistentTile<12, 2, 1>::SM == 2 && PersistentTile<12, 2, 1>::LS == 1, "tile table");
 static_assert(PersistentTile<12, 2, 2>::SM == 1 && PersistentTile<12, 2, 2>::LS == 2, "tile table");
@@ -289,8 +288,8 @@ const char* persistent_variant_name(const RnsConsts& rc, int v)
          "1 coefficient per thread, 4 primes per pass",
          "2 coefficients per thread, 2 primes per pass; lean NTT exchange addresses and reductions",
          "2 coefficients per thread, 2 primes per pass; inverse NTT with a warp-shuffle stage"},
-        {"1 coefficient per thread, 8 primes per pass", "1 coefficient per thread, 4 primes per pass",
-         "1 coefficient per thread, 2 primes per pass", "", ""},
+        {"tensor-core rounding, sums loaded after the product", "tensor-core rounding, sums loaded before the product",
+         "tensor-core rounding, plain inverse NTT", "", ""},
         {"2 coefficients per thread, 2 primes per pass", "2 coefficients per thread, 1 prime per pass",
          "1 coefficient per thread, 2 primes per pass", "", ""},
     };

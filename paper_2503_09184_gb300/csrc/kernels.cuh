@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "ntt.cuh"
+#include "round_mma.cuh"
 #include "worklist.h"
 
 template <int LOGN, int L>
@@ -232,6 +233,13 @@ SFHE_DEV void scale_round_b(const u32* x32, size_t stride, const RnsConsts& c, u
     scale_round_m<L, K, 1>(src, stride, c, dd);
 #pragma unroll
     for (int i = 0; i < L; i++) d[i] = dd[0][i];
+}
+
+// the same out of line, for the few coefficients that RoundMma cannot round
+template <int L, int K>
+__device__ __noinline__ void round_exact(const u32* x32, size_t stride, const RnsConsts& c, u64* d)
+{
+    scale_round_b<L, K>(x32, stride, c, d);
 }
 
 // ------------------------------------------------------------------------
@@ -672,8 +680,17 @@ template <int LOGN, int L, int V>
 struct PersistentTile {
     static constexpr int K = tensor_base_size(LOGN, L);
     static constexpr int R = NttGeom<LOGN>::T32::R;
+    // the scale-and-round on the tensor cores (round_mma.cuh has the reasons);
+    // variant 1 then loads an entry's sums so far before it waits for a
+    // tile's product instead of after, variant 2 takes the plain inverse NTT
+    static constexpr bool MMA = K > 16;  // round_on_tensor_cores
+    using RM = RoundMma<MMA ? L : 8, MMA ? K : 30>;
+    static constexpr int WGS = NttGeom<LOGN>::T32::NT / 128;  // groups of four warps, each with its tiles
+    static constexpr int TILE_COLS = RM::ACOLS + RM::NC, TMEM_COLS = WGS * TILE_COLS;
+    static_assert(!MMA || TMEM_COLS == 256 || TMEM_COLS == 512, "tensor memory of stage S");
+    static constexpr bool EARLY = V == 1;
     static constexpr int VS = V >= 3 ? 1 : V;  // the stage-S tile
-    static constexpr int NTT_FORM = V == 3 ? 1 : (V == 4 ? 2 : 0);
+    static constexpr int NTT_FORM = MMA ? (V == 2 ? 3 : 0) : (V == 3 ? 1 : (V == 4 ? 2 : 0));
     static constexpr int SMD = (K <= 16 && R <= 16) ? 2 : 1;
     static constexpr int SM = (VS == 2 && SMD == 2) ? 1 : SMD;
     static constexpr int LS = VS == 1 ? (L >= 2 ? L / 2 : L) : ((VS == 2 && SMD == 1) ? (L >= 4 ? L / 4 : L) : L);
@@ -712,7 +729,9 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
 {
     using CF = Cfg<LOGN, L>;
     using NQ = typename CF::NQ;
-    using NB = typename PersistentTile<LOGN, L, V>::NB;
+    using TL = PersistentTile<LOGN, L, V>;
+    using NB = typename TL::NB;
+    using RM = typename TL::RM;
     using PP = PersistentPlan<LOGN, L>;
     constexpr int N = NQ::N, NTH = NB::NT, K = CF::K, R = NB::R;
     constexpr int VT = NQ::NT / NTH;  // virtual threads of the 64-bit transforms per thread
@@ -721,7 +740,8 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
     u32* sm32 = reinterpret_cast<u32*>(sm);
     unsigned char* smb = reinterpret_cast<unsigned char*>(sm);
     __shared__ int s_entry;
-    __shared__ __align__(8) u64 mbar[2];
+    __shared__ __align__(8) u64 mbar[2], mma_bar[TL::WGS], row_bar[TL::WGS];
+    __shared__ u32 s_tmem;
     const int tid = threadIdx.x;
     u64* base = scratch + (size_t)blockIdx.x * scratch_stride;
     u64* cacc = base + (size_t)3 * L * N;                   // [2][N] u64, behind the sums [3][L][N]
@@ -741,6 +761,30 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
             fence_mbar_init();
         }
     }
+    // stage S on the tensor cores: its barriers (one pair per group of four
+    // warps; both are used once per tile, their phases go together) and tensor memory
+    u32 tmem = 0, mma_phase = 0;
+    if constexpr (TL::MMA) {
+        if (tid == 0) {
+            for (int i = 0; i < TL::WGS; i++) mbar_init(&mma_bar[i], 1), mbar_init(&row_bar[i], 4);
+            fence_mbar_init();
+        }
+        if (tid < 32) tmem_alloc<TL::TMEM_COLS>(&s_tmem);
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        tmem = s_tmem;
+    }
+    auto release_tmem = [&]() {  // by every thread, before the CTA leaves
+        if constexpr (TL::MMA) {
+            tc_fence_before();
+            __syncthreads();
+            if (tid < 32) {
+                tc_fence_after();
+                tmem_dealloc<TL::TMEM_COLS>(tmem);
+            }
+        }
+    };
     // bounded wait on mbarrier bi by every thread; false (in every thread) if
     // any thread's wait ran out
     auto wait_bar = [&](int bi) -> bool {
@@ -768,6 +812,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
             for (int bi = 0; bi < 2; bi++)
                 if (pend & (1u << bi)) mbar_wait(&mbar[bi], (phbits >> bi) & 1u, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
         }
+        release_tmem();
     };
 
     for (;;) {
@@ -799,8 +844,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
         // into the entry's sums, SM coefficients per thread at a time.  d0 and
         // d1 only need to be congruent (stage R reduces their sums), so they
         // stay in [0, 3 q_i); the digits of d2 must be canonical.
-        auto stage_s = [&](int pr) {
-            using TL = PersistentTile<LOGN, L, V>;
+        auto stage_s_cores = [&](int pr) {
             constexpr int SM = TL::SM, LS = TL::LS;
             constexpr bool HOIST = K <= 16;
             const bool fold = pr != 0 && (pr & 255) == 0;  // sums below 2^64: fold every 256 products
@@ -847,6 +891,74 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
 #pragma unroll 1
                 for (int p = 0; p < 2; p++) poly(p, k, std::true_type{});
                 poly(2, k, std::false_type{});
+            }
+        };
+        // The same on the tensor cores: d0 and d1 stay below 2^55.3.  The right
+        // operand is copied into the idle exchange buffers.  False (in some
+        // threads) if a matrix product did not complete within the wait bound.
+        auto stage_s_mma = [&](int pr) -> bool {
+            const bool fold = pr != 0 && pr % 255 == 0;  // sums below 2^54.1 + 255 2^55.3 < 2^64
+            const int wg = tid >> 7, row = tid & 127;
+            constexpr int PT = N / 128, NTILE = 3 * PT / TL::WGS;
+            static_assert(PT % TL::WGS == 0 && RM::BYTES <= (int)PP::EXB, "tiles of stage S");
+            for (int w = tid; w < RM::BYTES / 16; w += NTH)
+                reinterpret_cast<uint4*>(smb)[w] = __ldg(reinterpret_cast<const uint4*>(c.mm_b) + w);
+            fence_proxy_async();
+            __syncthreads();
+            const u32 a = tmem + wg * TL::TILE_COLS, d = a + RM::ACOLS, lane = (u32)((tid >> 5) & 3) << 21;
+            bool alive = true;
+#pragma unroll 1
+            for (int j = 0; j < NTILE; j++) {
+                const int t = j * TL::WGS + wg, p = t / PT, e = t % PT * 128 + row;
+                const u32* src = T + (size_t)p * K * N + e;
+                u64* sum = acc + (size_t)p * L * N + e;
+                RM::store_row(src, N, a + lane);
+                tc_fence_before();
+                __syncwarp();
+                // the group's first warp waits for the four warps' rows
+                if ((row & 31) == 0) mbar_arrive(&row_bar[wg]);
+                if (row < 32) {
+                    if (alive) alive = mbar_wait(&row_bar[wg], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
+                    if (row == 0) {
+                        tc_fence_after();
+                        RM::issue(d, a, smem_addr(smb));
+                        mma_commit(&mma_bar[wg]);
+                    }
+                }
+                u64 prev[L], w[L];
+                auto load_prev = [&]() {
+#pragma unroll
+                    for (int i = 0; i < L; i++) prev[i] = pr == 0 ? 0 : sum[(size_t)i * N];
+                };
+                if constexpr (TL::EARLY) load_prev();
+                if (alive) alive = mbar_wait(&mma_bar[wg], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
+                mma_phase ^= 1u;
+                tc_fence_after();
+                const bool ok = RM::load_row(d + lane, c, w);
+                tc_fence_before();
+                if constexpr (!TL::EARLY) load_prev();
+                if (p == 2) {
+#pragma unroll
+                    for (int i = 0; i < L; i++) w[i] = pm_canon((i64)w[i], c.m[i].q);
+                }
+                if (!ok) round_exact<L, K>(src, N, c, w);  // about one in 2^26
+                if (fold && p < 2) {
+#pragma unroll
+                    for (int i = 0; i < L; i++) prev[i] = (u64)pm_fold_u(prev[i], pm_c(c.m[i].q));
+                }
+#pragma unroll
+                for (int i = 0; i < L; i++) sum[(size_t)i * N] = prev[i] + w[i];
+            }
+            return alive;
+        };
+        // stage S and the barrier behind it; false (in every thread) if a wait ran out
+        auto stage_s = [&](int pr) -> bool {
+            if constexpr (TL::MMA) {
+                return !__syncthreads_or(!stage_s_mma(pr));
+            } else {
+                stage_s_cores(pr);
+                __syncthreads();
+                return true;
             }
         };
         if constexpr (PP::STAGED) {
@@ -914,8 +1026,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                     }
                     if (k == K - 1) {
                         __syncthreads();
-                        stage_s(pr);
-                        __syncthreads();
+                        if (!stage_s(pr)) {
+                            abort_cta();
+                            return;
+                        }
                     }
                 }
             } else {
@@ -1024,8 +1138,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                     }
                 }
                 __syncthreads();
-                stage_s(g);
-                __syncthreads();
+                if (!stage_s(g)) {
+                    abort_cta();
+                    return;
+                }
             }
             }
         } else {
@@ -1081,8 +1197,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                         }
                     }
                     __syncthreads();
-                    stage_s(pr);
-                    __syncthreads();
+                    if (!stage_s(pr)) {
+                        abort_cta();
+                        return;
+                    }
                 }
             } else if constexpr (GROUPED && PP::STAGED2) {
                 // the same rounds, each over the group's products (the
@@ -1149,8 +1267,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                         }
                     }
                     __syncthreads();
-                    stage_s(g);
-                    __syncthreads();
+                    if (!stage_s(g)) {
+                        abort_cta();
+                        return;
+                    }
                 }
             } else if constexpr (!GROUPED) {
                 for (int pr = 0; pr < en.count; pr++) {
@@ -1174,8 +1294,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                         }
                     }
                     __syncthreads();
-                    stage_s(pr);
-                    __syncthreads();
+                    if (!stage_s(pr)) {
+                        abort_cta();
+                        return;
+                    }
                 }
             } else {
             for (int g = 0; g * G < en.count; g++) {
@@ -1204,8 +1326,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                     }
                 }
                 __syncthreads();
-                stage_s(g);
-                __syncthreads();
+                if (!stage_s(g)) {
+                    abort_cta();
+                    return;
+                }
             }
             }
         }
@@ -1336,4 +1460,5 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
         // the slots are refilled by bulk copies (async proxy) for the next entry
         if constexpr (PP::STAGED || PP::STAGED2) fence_proxy_async();
     }
+    release_tmem();
 }

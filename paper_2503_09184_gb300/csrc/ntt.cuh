@@ -126,7 +126,8 @@ struct Arith32 {
 
 // FORM_ picks code forms of the same transform (the run-time tuner's NTT
 // candidates; every form computes the same values): 0 the default, 1 the
-// lean forms at every size, 2 the inverse's shuffle stage where it applies.
+// lean forms at every size, 2 the inverse's shuffle stage where it applies, 3
+// the plain forms at every size.
 template <int LOGN_, int LOGR_, typename A, int FORM_ = 0>
 struct NttT {
     using W = typename A::W;
@@ -144,7 +145,7 @@ struct NttT {
     // kernel sits at the register limit; so by default they are taken from
     // N = 16384 (form 1 takes them everywhere).
     static constexpr int FORM = FORM_;
-    static constexpr bool LEAN = LOGN >= 14 || FORM == 1;
+    static constexpr bool LEAN = (LOGN >= 14 && FORM != 3) || FORM == 1;
     // Inverse with one stage more than whole passes (32-bit words, form 2):
     // the stage after the first pass pairs each thread with its neighbour
     // (tid ^ 1) and runs on warp shuffles, so the passes are LOGR + 1, LOGR,

@@ -108,6 +108,17 @@ struct RnsConsts {
     u64 r_w[SFHE_MAX_K][SFHE_MAX_L + 1];          // r_k as words (exact decision)
     u64 rB_w[SFHE_MAX_L + 1];                     // r_B as words
 
+    // the rounding on the tensor cores (round_mma.cuh): right operand (fp16,
+    // device memory), the constant of v, the constants of F's two halves and
+    // -r_B 2^54 / Q split at bit 27, [-alpha_B]_{q_i} split at bit 27, and per
+    // prime the constant that the digits' offsets leave
+    const unsigned short* mm_b;
+    u32 mm_vc, mm_p9, mm_p18, mm_p27;  // the powers are 2^9, 2^18, 2^27
+    int mm_rb0n, mm_rb1n;
+    u64 mm_g0, mm_g1;
+    u32 mm_nab_lo[SFHE_MAX_L], mm_nab_hi[SFHE_MAX_L];
+    u64 mm_cq[SFHE_MAX_L];
+
     // products per rounding in the grouped accumulate-then-round mode:
     // floor(B / (2 N Q^2)), at most 1024
     int lazy_group;
