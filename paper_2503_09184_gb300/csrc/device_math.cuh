@@ -298,6 +298,17 @@ SFHE_DEV u64 sample_uniform(u64 key, u64 slot, u64 q, int* fail)
     *fail = 1;
     return 0;
 }
+// the same for q = 2^54 - c, c < 2^23: floor(2^64 / q) = 1024, and the
+// reduction is one fold (no 64-bit division, which took most of encryption)
+SFHE_DEV u64 sample_uniform54(u64 key, u64 slot, u64 q, int* fail)
+{
+    for (u64 r = 0; r < 16; r++) {
+        const u64 w = sm_word(key, slot * 16 + r);
+        if (w < q << 10) return csub((u64)pm_fold_u(w, pm_c(q)), q);
+    }
+    *fail = 1;
+    return 0;
+}
 SFHE_DEV int sample_ternary(u64 key, u64 slot, int* fail)
 {
     u64 lim = (~0ULL / 3) * 3;
@@ -315,12 +326,16 @@ SFHE_DEV int sample_gauss(u64 key, u64 slot, const u64* cdt)
 {
     u64 w = sm_word(key, slot * 16);
     u64 u = w >> 1;
+    // the table ascends: the count of entries not above u, without a loop
+    // whose length is the warp's longest
     int k = 0;
-    while (k < 19 && u >= cdt[k]) k++;
-    if (k == 0) return 0;
+#pragma unroll
+    for (int j = 0; j < 19; j++) k += u >= cdt[j];
     return (w & 1) ? -k : k;
 }
-// signed small integer to its residue mod q
+// residue mod q of an integer between -q and q
+SFHE_DEV u64 small_residue(int v, u64 q) { return v < 0 ? q - (u64)(-v) : (u64)v; }
+// signed integer to its residue mod q
 SFHE_DEV u64 to_residue(long long v, u64 q)
 {
     if (v >= 0) return (u64)v % q;

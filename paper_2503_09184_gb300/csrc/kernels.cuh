@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_keygen_secret(const __
         const int e = NT_::fwd_in_idx(v, tid);
         const int s = sample_ternary(key, (u64)e, &fail);
         if (l == 0) s_coeff[e] = (signed char)s;
-        x[v] = to_residue(s, m.q);
+        x[v] = small_residue(s, m.q);
     }
     NT_::forward(x, sm, tid, c.tw + (size_t)l * 4 * NT_::N, m.q);
     NT_::run_to_lane(x, sm, tid);
@@ -392,31 +392,32 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_keygen_rlk(const __gri
     int fail = 0;
     const u64 ka = sm_key(c.seed, SFHE_DOM_RLK_A, (u64)j, 0, 0);
     const u64 ke = sm_key(c.seed, SFHE_DOM_RLK_E, (u64)j, 0, 0);
-    u64 a[NT_::R], e[NT_::R];
-#pragma unroll
-    for (int v = 0; v < NT_::R; v++) {
-        const int k = NT_::fwd_in_idx(v, tid);
-        a[v] = sample_uniform(ka, (u64)i * N + k, m.q, &fail);
-        e[v] = to_residue(sample_gauss(ke, (u64)k, c.cdt), m.q);
-    }
-    NT_::forward(a, sm, tid, tw, m.q);
-    NT_::forward(e, sm, tid, tw, m.q);
     u64* b_out = rlk + (((size_t)j * 2 + 0) * L + i) * N;
     u64* a_out = rlk + (((size_t)j * 2 + 1) * L + i) * N;
     ulonglong2* bp_out = reinterpret_cast<ulonglong2*>(rlk_pm) + (((size_t)j * 2 + 0) * L + i) * N;
     ulonglong2* ap_out = reinterpret_cast<ulonglong2*>(rlk_pm) + (((size_t)j * 2 + 1) * L + i) * N;
+    // one polynomial in registers at a time; a thread reads back its own words of a
+    u64 x[NT_::R];
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = sample_uniform54(ka, (u64)i * N + NT_::fwd_in_idx(v, tid), m.q, &fail);
+    NT_::forward(x, sm, tid, tw, m.q);
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) {
+        const u64 av = pm_canon((i64)x[v], m.q);
+        a_out[NT_::run_idx(v, tid)] = av;
+        ap_out[NT_::lane_idx(v, tid)] = make_ulonglong2(pm_pack(av, m.q), pm_pack(barrett(av >> 32, av << 32, m), m.q));
+    }
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = small_residue(sample_gauss(ke, (u64)NT_::fwd_in_idx(v, tid), c.cdt), m.q);
+    NT_::forward(x, sm, tid, tw, m.q);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::run_idx(v, tid);
-        const u64 av = pm_canon((i64)a[v], m.q), ev = pm_canon((i64)e[v], m.q);
         const u64 sv = s_ntt[(size_t)i * N + k];
-        u64 bv = sub_mod(ev, mul_mod(av, sv, m), m.q);
+        u64 bv = sub_mod(pm_canon((i64)x[v], m.q), mul_mod(a_out[k], sv, m), m.q);
         if (i == j) bv = add_mod(bv, mul_mod(sv, sv, m), m.q);
         b_out[k] = bv;
-        a_out[k] = av;
-        const int kl = NT_::lane_idx(v, tid);
-        bp_out[kl] = make_ulonglong2(pm_pack(bv, m.q), pm_pack(barrett(bv >> 32, bv << 32, m), m.q));
-        ap_out[kl] = make_ulonglong2(pm_pack(av, m.q), pm_pack(barrett(av >> 32, av << 32, m), m.q));
+        bp_out[NT_::lane_idx(v, tid)] = make_ulonglong2(pm_pack(bv, m.q), pm_pack(barrett(bv >> 32, bv << 32, m), m.q));
     }
     if (fail) atomicExch(err, 1);
 }
@@ -441,27 +442,29 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_encrypt(const __grid_c
     long long mt = vals[n] % (long long)c.t;
     if (mt < 0) mt += (long long)c.t;
     int fail = 0;
-    u64 a[NT_::R], e[NT_::R];
+    u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
+    u64* c1 = c0 + (size_t)L * N;
+    // one polynomial in registers at a time; a thread reads back its own words of c1
+    u64 x[NT_::R];
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = sample_uniform54(ka, (u64)l * N + NT_::fwd_in_idx(v, tid), m.q, &fail);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) c1[NT_::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::fwd_in_idx(v, tid);
-        a[v] = sample_uniform(ka, (u64)l * N + k, m.q, &fail);
-        u64 ev = to_residue(sample_gauss(ke, (u64)k, c.cdt), m.q);
+        u64 ev = small_residue(sample_gauss(ke, (u64)k, c.cdt), m.q);
         if (k == 0) ev = add_mod(ev, mul_mod(c.delta_q[l], (u64)mt, m), m.q);
-        e[v] = ev;
+        x[v] = ev;
     }
-    NT_::forward(a, sm, tid, tw, m.q);
-    NT_::forward(e, sm, tid, tw, m.q);
-    u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
-    u64* c1 = c0 + (size_t)L * N;
-    NT_::run_to_lane(a, sm, tid);
-    NT_::run_to_lane(e, sm, tid);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::lane_idx(v, tid);
-        const u64 av = pm_canon((i64)a[v], m.q);
-        c0[k] = sub_mod(pm_canon((i64)e[v], m.q), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
-        c1[k] = av;
+        c0[k] = sub_mod(pm_canon((i64)x[v], m.q), mul_mod(c1[k], s_ntt[(size_t)l * N + k], m), m.q);
     }
     if (fail) atomicExch(err, 1);
 }

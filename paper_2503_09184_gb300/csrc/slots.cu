@@ -55,32 +55,35 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_galois_keygen(const __
     int fail = 0;
     const u64 ka = sm_key(c.seed, SFHE_DOM_GAL_A, (u64)g, (u64)j, 0);
     const u64 ke = sm_key(c.seed, SFHE_DOM_GAL_E, (u64)g, (u64)j, 0);
-    u64 a[NT_::R], e[NT_::R];
-#pragma unroll
-    for (int v = 0; v < NT_::R; v++) {
-        const int k = NT_::fwd_in_idx(v, tid);
-        a[v] = sample_uniform(ka, (u64)i * N + k, m.q, &fail);
-        e[v] = to_residue(sample_gauss(ke, (u64)k, c.cdt), m.q);
-    }
-    NT_::forward(a, sm, tid, tw, m.q);
-    NT_::forward(e, sm, tid, tw, m.q);
     u64* b_out = key + (((size_t)j * 2 + 0) * L + i) * N;
     u64* a_out = key + (((size_t)j * 2 + 1) * L + i) * N;
     u64* bs_out = key_sh + (((size_t)j * 2 + 0) * L + i) * N;
     u64* as_out = key_sh + (((size_t)j * 2 + 1) * L + i) * N;
     const u64* s = s_ntt + (size_t)i * N;
-    NT_::run_to_lane(a, sm, tid);
-    NT_::run_to_lane(e, sm, tid);
+    // one polynomial in registers at a time; a thread reads back its own words of a
+    u64 x[NT_::R];
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = sample_uniform54(ka, (u64)i * N + NT_::fwd_in_idx(v, tid), m.q, &fail);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::lane_idx(v, tid);
-        const u64 av = pm_canon((i64)a[v], m.q), ev = pm_canon((i64)e[v], m.q);
-        u64 bv = sub_mod(ev, mul_mod(av, s[k], m), m.q);
+        const u64 av = pm_canon((i64)x[v], m.q);
+        a_out[k] = av;
+        as_out[k] = (u64)(((unsigned __int128)av << 64) / m.q);
+    }
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = small_residue(sample_gauss(ke, (u64)NT_::fwd_in_idx(v, tid), c.cdt), m.q);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) {
+        const int k = NT_::lane_idx(v, tid);
+        u64 bv = sub_mod(pm_canon((i64)x[v], m.q), mul_mod(a_out[k], s[k], m), m.q);
         if (i == j) bv = add_mod(bv, s[galois_src<LOGN>(k, g)], m.q);
         b_out[k] = bv;
-        a_out[k] = av;
         bs_out[k] = (u64)(((unsigned __int128)bv << 64) / m.q);
-        as_out[k] = (u64)(((unsigned __int128)av << 64) / m.q);
     }
     if (fail) atomicExch(err, 1);
 }
@@ -105,27 +108,29 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_encrypt_poly(const __g
     const u64 ke = sm_key(c.seed, SFHE_DOM_ENC_E, matrix_id, row, col);
     const long long* msg = polys + (size_t)n * N;
     int fail = 0;
-    u64 a[NT_::R], e[NT_::R];
+    u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
+    u64* c1 = c0 + (size_t)L * N;
+    // one polynomial in registers at a time; a thread reads back its own words of c1
+    u64 x[NT_::R];
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) x[v] = sample_uniform54(ka, (u64)l * N + NT_::fwd_in_idx(v, tid), m.q, &fail);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
+#pragma unroll
+    for (int v = 0; v < NT_::R; v++) c1[NT_::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::fwd_in_idx(v, tid);
-        a[v] = sample_uniform(ka, (u64)l * N + k, m.q, &fail);
         long long mt = msg[k] % (long long)c.t;
         if (mt < 0) mt += (long long)c.t;
-        e[v] = add_mod(to_residue(sample_gauss(ke, (u64)k, c.cdt), m.q), mul_mod(c.delta_q[l], (u64)mt, m), m.q);
+        x[v] = add_mod(small_residue(sample_gauss(ke, (u64)k, c.cdt), m.q), mul_mod(c.delta_q[l], (u64)mt, m), m.q);
     }
-    NT_::forward(a, sm, tid, tw, m.q);
-    NT_::forward(e, sm, tid, tw, m.q);
-    u64* c0 = ct + ((size_t)n * 2 * L + l) * N;
-    u64* c1 = c0 + (size_t)L * N;
-    NT_::run_to_lane(a, sm, tid);
-    NT_::run_to_lane(e, sm, tid);
+    NT_::forward(x, sm, tid, tw, m.q);
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::lane_idx(v, tid);
-        const u64 av = pm_canon((i64)a[v], m.q);
-        c0[k] = sub_mod(pm_canon((i64)e[v], m.q), mul_mod(av, s_ntt[(size_t)l * N + k], m), m.q);
-        c1[k] = av;
+        c0[k] = sub_mod(pm_canon((i64)x[v], m.q), mul_mod(c1[k], s_ntt[(size_t)l * N + k], m), m.q);
     }
     if (fail) atomicExch(err, 1);
 }
