@@ -261,7 +261,7 @@ extern "C" sfhe_status sfhe_ctx_create(const sfhe_params* params, uint64_t seed,
     cdt_table(params->sigma, rc.cdt);
 
     std::vector<uint64_t> tw((size_t)rc.L * 4 * N);
-    for (int i = 0; i < rc.L; i++) twiddles_pm(rc.m[i].q, N, tw.data() + (size_t)i * 4 * N, &rc.ninv_pm[i], &rc.wlast_pm[i]);
+    for (int i = 0; i < rc.L; i++) twiddles_pm(rc.m[i].q, N, 16, tw.data() + (size_t)i * 4 * N, &rc.ninv_pm[i], &rc.wlast_pm[i]);
     std::vector<uint32_t> twb((size_t)rc.K * 4 * N);
     for (int k = 0; k < rc.K; k++)
         twiddles32(rc.mb[k].b, N, twb.data() + (size_t)k * 4 * N, &rc.ninv_b[k], &rc.wlast_b[k]);

@@ -18,6 +18,8 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include <type_traits>
+
 #include "../../include/sfhe.h"
 #include "api_internal.h"
 #include "host_math.h"
@@ -43,6 +45,8 @@ struct CkksConsts {
     ModG m[CK_MAX];
     const u64* tw;  // [L + 1][4][N]
     ShoupC ninv[CK_MAX], wlast[CK_MAX];
+    PmC ninv_pm[CK_MAX], wlast_pm[CK_MAX];
+    int pm;  // CkGeom's PM: the tables are twiddles_pm's
     ShoupC pinv[CK_MAX];               // P^-1 mod q_i
     ShoupC qinv[CK_MAX][CK_MAX];       // q_l^-1 mod q_i (i < l)
     u64 cdt[20];
@@ -83,13 +87,26 @@ SFHE_DEV int galois_src_ck(int i, u32 g)
     return (int)(__brev((unsigned)((f - 1) >> 1)) >> (32 - LOGN));
 }
 
-template <int LOGN>
+// PM: every prime is 2^n - c with 32 < n <= 54 and c < 2^23 (pm_fits; the
+// paper's sizes are), and the transforms multiply as the 54-bit ones do
+// (ArithPm); else Shoup's form.  The chunked 8 x 8 x 8 product at N = 8192
+// (GB300): 4.57 ms with it and coalesced words, 6.15 without.
+template <int LOGN, bool PM>
 struct CkGeom {
-    using T = NttT<LOGN, 4, Arith64>;
-};
-template <>
-struct CkGeom<6> {
-    using T = NttT<6, 2, Arith64>;  // 16 threads at N = 64
+    using A = std::conditional_t<PM, ArithPm<true>, Arith64>;
+    using T = NttT<LOGN, LOGN == 6 ? 2 : 4, A>;  // 16 threads at N = 64
+    // a valid forward input from any 64-bit word
+    SFHE_DEV static u64 fwd_in(u64 x, const ModG& m)
+    {
+        if constexpr (PM) return (u64)pm_fold_any_u(x, pm_c_any(m.q), pm_bits(m.q));
+        else return reduce_g(x, m);
+    }
+    // canonical residue of a transform's output
+    SFHE_DEV static u64 canon(u64 x, const ModG& m)
+    {
+        if constexpr (PM) return pm_canon_any((i64)x, m.q);
+        else return reduce_g(x, m);
+    }
 };
 
 // ------------------------------------------------------------------ kernels ---
@@ -101,13 +118,14 @@ struct PrimeList {
     int idx[CK_MAX];
 };
 
-template <int LOGN>
-__global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ntt(const __grid_constant__ CkksConsts c, int inverse,
+template <int LOGN, bool PM>
+__global__ void __launch_bounds__(CkGeom<LOGN, PM>::T::NT) k_ck_ntt(const __grid_constant__ CkksConsts c, int inverse,
                                                                 const u64* in, size_t in_gstride, size_t in_lstride,
                                                                 u64* out, size_t out_gstride, size_t out_lstride,
                                                                 PrimeList pl)
 {
-    using NT_ = typename CkGeom<LOGN>::T;
+    using GE = CkGeom<LOGN, PM>;
+    using NT_ = typename GE::T;
     extern __shared__ u64 sm[];
     const int l = blockIdx.x, g = blockIdx.y, tid = threadIdx.x, pi = pl.idx[l];
     const ModG m = c.m[pi];
@@ -117,29 +135,36 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ntt(const __grid_con
     u64 x[NT_::R];
     if (!inverse) {
 #pragma unroll
-        for (int v = 0; v < NT_::R; v++) x[v] = reduce_g(src[NT_::fwd_in_idx(v, tid)], m);
+        for (int v = 0; v < NT_::R; v++) x[v] = GE::fwd_in(src[NT_::fwd_in_idx(v, tid)], m);
         NT_::forward(x, sm, tid, tw, m.q);
+        NT_::run_to_lane(x, sm, tid);
 #pragma unroll
-        for (int v = 0; v < NT_::R; v++) dst[NT_::run_idx(v, tid)] = reduce_g(x[v], m);
+        for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = GE::canon(x[v], m);
     } else {
 #pragma unroll
-        for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::run_idx(v, tid)];
-        NT_::inverse(x, sm, tid, tw, m.q, c.ninv[pi].w, c.ninv[pi].ws, c.wlast[pi].w, c.wlast[pi].ws);
+        for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::lane_idx(v, tid)];
+        NT_::lane_to_run(x, sm, tid);
+        if constexpr (PM)
+            NT_::inverse(x, sm, tid, tw, m.q, c.ninv_pm[pi].w, c.ninv_pm[pi].w2, c.wlast_pm[pi].w, c.wlast_pm[pi].w2);
+        else
+            NT_::inverse(x, sm, tid, tw, m.q, c.ninv[pi].w, c.ninv[pi].ws, c.wlast[pi].w, c.wlast[pi].ws);
 #pragma unroll
-        for (int v = 0; v < NT_::R; v++) dst[NT_::inv_out_idx(v, tid)] = csub(x[v], m.q);
+        for (int v = 0; v < NT_::R; v++)
+            dst[NT_::inv_out_idx(v, tid)] = PM ? GE::canon(x[v], m) : csub(x[v], m.q);
     }
 }
 
 // Forward transforms of centred residues: block (t, g): input polynomial g
 // is canonical mod prime `from`, its centred representatives are taken mod
 // prime pl.idx[t] and transformed.  (The rescale and the division by P.)
-template <int LOGN>
-__global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ntt_centred(const __grid_constant__ CkksConsts c,
+template <int LOGN, bool PM>
+__global__ void __launch_bounds__(CkGeom<LOGN, PM>::T::NT) k_ck_ntt_centred(const __grid_constant__ CkksConsts c,
                                                                         int from, const u64* in, size_t in_gstride,
                                                                         u64* out, size_t out_gstride,
                                                                         size_t out_lstride, PrimeList pl)
 {
-    using NT_ = typename CkGeom<LOGN>::T;
+    using GE = CkGeom<LOGN, PM>;
+    using NT_ = typename GE::T;
     extern __shared__ u64 sm[];
     const int t = blockIdx.x, g = blockIdx.y, tid = threadIdx.x, pi = pl.idx[t];
     const ModG m = c.m[pi];
@@ -150,17 +175,19 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ntt_centred(const __
     for (int v = 0; v < NT_::R; v++) x[v] = centred_mod(src[NT_::fwd_in_idx(v, tid)], p, m);
     NT_::forward(x, sm, tid, c.tw + (size_t)pi * 4 * NT_::N, m.q);
     u64* dst = out + g * out_gstride + (size_t)t * out_lstride;
+    NT_::run_to_lane(x, sm, tid);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) dst[NT_::run_idx(v, tid)] = reduce_g(x[v], m);
+    for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = GE::canon(x[v], m);
 }
 
 // the secret: ternary coefficients (stream (seed, 1, 0, 0, 0), slot k) mod
 // every prime, NTT form; block (prime t)
-template <int LOGN>
-__global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_secret(const __grid_constant__ CkksConsts c, u64* s_ntt,
+template <int LOGN, bool PM>
+__global__ void __launch_bounds__(CkGeom<LOGN, PM>::T::NT) k_ck_secret(const __grid_constant__ CkksConsts c, u64* s_ntt,
                                                                    int* err)
 {
-    using NT_ = typename CkGeom<LOGN>::T;
+    using GE = CkGeom<LOGN, PM>;
+    using NT_ = typename GE::T;
     extern __shared__ u64 sm[];
     const int t = blockIdx.x, tid = threadIdx.x;
     const ModG m = c.m[t];
@@ -174,7 +201,7 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_secret(const __grid_
     }
     NT_::forward(x, sm, tid, c.tw + (size_t)t * 4 * NT_::N, m.q);
 #pragma unroll
-    for (int v = 0; v < NT_::R; v++) s_ntt[(size_t)t * NT_::N + NT_::run_idx(v, tid)] = reduce_g(x[v], m);
+    for (int v = 0; v < NT_::R; v++) s_ntt[(size_t)t * NT_::N + NT_::run_idx(v, tid)] = GE::canon(x[v], m);
     if (fail) atomicExch(err, 1);
 }
 
@@ -182,12 +209,13 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_secret(const __grid_
 // a uniform (stream (seed, 9, g, j, 0), slot t N + k), e Gaussian (stream
 // (seed, 10, g, j, 0), slot k), b = -a s + e + [t = j] P w; NTT form with
 // Shoup companions; layout [L digit][2 (b, a)][L + 1 prime][N].
-template <int LOGN>
-__global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ksk(const __grid_constant__ CkksConsts c,
+template <int LOGN, bool PM>
+__global__ void __launch_bounds__(CkGeom<LOGN, PM>::T::NT) k_ck_ksk(const __grid_constant__ CkksConsts c,
                                                                 const u64* s_ntt, u32 g, u64* key, u64* key_sh,
                                                                 int* err)
 {
-    using NT_ = typename CkGeom<LOGN>::T;
+    using GE = CkGeom<LOGN, PM>;
+    using NT_ = typename GE::T;
     constexpr int N = NT_::N;
     extern __shared__ u64 sm[];
     const int t = blockIdx.x, j = blockIdx.y, tid = threadIdx.x, L = c.L;
@@ -212,7 +240,7 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ksk(const __grid_con
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::run_idx(v, tid);
-        const u64 av = reduce_g(a[v], m), ev = reduce_g(e[v], m);
+        const u64 av = GE::canon(a[v], m), ev = GE::canon(e[v], m);
         u64 bv = sub_mod(ev, mulmod_g(av, s[k], m), m.q);
         if (t == j) {
             const u64 w = g == 0 ? mulmod_g(s[k], s[k], m) : s[galois_src_ck<LOGN>(k, g)];
@@ -229,12 +257,13 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_ksk(const __grid_con
 // Encryption of integer plaintext polynomials at the top level, block
 // (limb i, ciphertext n): c1 = a (stream (seed, 11, id, row, col), slot
 // i N + k), c0 = -a s + e + m (e from stream (seed, 12, id, row, col), slot k).
-template <int LOGN>
-__global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_encrypt(const __grid_constant__ CkksConsts c,
+template <int LOGN, bool PM>
+__global__ void __launch_bounds__(CkGeom<LOGN, PM>::T::NT) k_ck_encrypt(const __grid_constant__ CkksConsts c,
                                                                     const u64* s_ntt, const long long* polys,
                                                                     const int* coords, u64 matrix_id, u64* ct, int* err)
 {
-    using NT_ = typename CkGeom<LOGN>::T;
+    using GE = CkGeom<LOGN, PM>;
+    using NT_ = typename GE::T;
     constexpr int N = NT_::N;
     extern __shared__ u64 sm[];
     const int i = blockIdx.x, n = blockIdx.y, tid = threadIdx.x, L = c.L;
@@ -262,8 +291,8 @@ __global__ void __launch_bounds__(CkGeom<LOGN>::T::NT) k_ck_encrypt(const __grid
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) {
         const int k = NT_::run_idx(v, tid);
-        const u64 av = reduce_g(a[v], m);
-        c0[k] = sub_mod(reduce_g(e[v], m), mulmod_g(av, s[k], m), m.q);
+        const u64 av = GE::canon(a[v], m);
+        c0[k] = sub_mod(GE::canon(e[v], m), mulmod_g(av, s[k], m), m.q);
         c1[k] = av;
     }
     if (fail) atomicExch(err, 1);
@@ -494,9 +523,9 @@ PrimeList one_prime(int i)
 }
 
 template <int LOGN>
-size_t ck_smem() { return (size_t)CkGeom<LOGN>::T::SMEM_WORDS * 8; }
+size_t ck_smem() { return (size_t)CkGeom<LOGN, true>::T::SMEM_WORDS * 8; }
 template <int LOGN>
-int ck_nt() { return CkGeom<LOGN>::T::NT; }
+int ck_nt() { return CkGeom<LOGN, true>::T::NT; }
 
 template <typename K>
 cudaError_t ck_allow(K* kernel, size_t bytes)
@@ -504,6 +533,14 @@ cudaError_t ck_allow(K* kernel, size_t bytes)
     if (bytes <= 48 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+
+// the transform kernels of a context: ring degree and arithmetic
+#define CK_DISPATCH_NTT(c_, ...)                                                                 \
+    if ((c_).logN != 6 && (c_).logN != 13) return cudaErrorInvalidValue;                         \
+    if ((c_).logN == 6 && (c_).pm) { constexpr int LG = 6; constexpr bool PM = true; __VA_ARGS__; }    \
+    else if ((c_).logN == 6) { constexpr int LG = 6; constexpr bool PM = false; __VA_ARGS__; }         \
+    else if ((c_).pm) { constexpr int LG = 13; constexpr bool PM = true; __VA_ARGS__; }          \
+    else { constexpr int LG = 13; constexpr bool PM = false; __VA_ARGS__; }
 
 #define CK_DISPATCH(logN, ...)                       \
     switch (logN) {                                  \
@@ -516,10 +553,10 @@ cudaError_t ntt(const CkksConsts& c, bool inverse, const u64* in, size_t in_g, s
                 size_t out_l, PrimeList pl, int nl, int ng, cudaStream_t s)
 {
     if (nl <= 0 || ng <= 0) return cudaSuccess;
-    CK_DISPATCH(c.logN, {
-        cudaError_t e = ck_allow(k_ck_ntt<LG>, ck_smem<LG>());
+    CK_DISPATCH_NTT(c, {
+        cudaError_t e = ck_allow(k_ck_ntt<LG, PM>, ck_smem<LG>());
         if (e != cudaSuccess) return e;
-        k_ck_ntt<LG><<<dim3(nl, ng), ck_nt<LG>(), ck_smem<LG>(), s>>>(c, inverse ? 1 : 0, in, in_g, in_l, out, out_g,
+        k_ck_ntt<LG, PM><<<dim3(nl, ng), ck_nt<LG>(), ck_smem<LG>(), s>>>(c, inverse ? 1 : 0, in, in_g, in_l, out, out_g,
                                                                      out_l, pl);
         return cudaGetLastError();
     });
@@ -529,10 +566,10 @@ cudaError_t ntt_centred(const CkksConsts& c, int from, const u64* in, size_t in_
                         size_t out_l, PrimeList pl, int nt, int ng, cudaStream_t s)
 {
     if (nt <= 0 || ng <= 0) return cudaSuccess;
-    CK_DISPATCH(c.logN, {
-        cudaError_t e = ck_allow(k_ck_ntt_centred<LG>, ck_smem<LG>());
+    CK_DISPATCH_NTT(c, {
+        cudaError_t e = ck_allow(k_ck_ntt_centred<LG, PM>, ck_smem<LG>());
         if (e != cudaSuccess) return e;
-        k_ck_ntt_centred<LG><<<dim3(nt, ng), ck_nt<LG>(), ck_smem<LG>(), s>>>(c, from, in, in_g, out, out_g, out_l,
+        k_ck_ntt_centred<LG, PM><<<dim3(nt, ng), ck_nt<LG>(), ck_smem<LG>(), s>>>(c, from, in, in_g, out, out_g, out_l,
                                                                              pl);
         return cudaGetLastError();
     });
@@ -590,10 +627,10 @@ extern "C" void sfhe_ckks_ctx_destroy(sfhe_ckks_ctx* c)
 static sfhe_status ckks_keygen(sfhe_ckks_ctx* c, u32 g, u64* key, u64* key_sh, cudaStream_t s)
 {
     auto launch = [&]() -> cudaError_t {
-        CK_DISPATCH(c->cc.logN, {
-            cudaError_t e = ck_allow(k_ck_ksk<LG>, ck_smem<LG>());
+        CK_DISPATCH_NTT(c->cc, {
+            cudaError_t e = ck_allow(k_ck_ksk<LG, PM>, ck_smem<LG>());
             if (e != cudaSuccess) return e;
-            k_ck_ksk<LG><<<dim3(c->cc.L + 1, c->cc.L), ck_nt<LG>(), ck_smem<LG>(), s>>>(c->cc, c->d_s, g, key, key_sh,
+            k_ck_ksk<LG, PM><<<dim3(c->cc.L + 1, c->cc.L), ck_nt<LG>(), ck_smem<LG>(), s>>>(c->cc, c->d_s, g, key, key_sh,
                                                                                        c->d_err);
             return cudaGetLastError();
         });
@@ -662,7 +699,13 @@ extern "C" sfhe_status sfhe_ckks_ctx_create(const sfhe_ckks_params* params, uint
     }
     sfhe::cdt_table(params->sigma > 0 ? params->sigma : 3.2, cc.cdt);
     std::vector<uint64_t> tw((size_t)(L + 1) * 4 * N);
-    for (uint32_t i = 0; i <= L; i++) sfhe::twiddles(cc.m[i].q, N, tw.data() + (size_t)i * 4 * N, &cc.ninv[i], &cc.wlast[i]);
+    cc.pm = 1;
+    for (uint32_t i = 0; i <= L; i++) cc.pm &= sfhe::pm_fits(cc.m[i].q) ? 1 : 0;
+    for (uint32_t i = 0; i <= L; i++) {
+        uint64_t* t = tw.data() + (size_t)i * 4 * N;
+        if (cc.pm) sfhe::twiddles_pm(cc.m[i].q, N, N == 64 ? 4 : 16, t, &cc.ninv_pm[i], &cc.wlast_pm[i]);
+        else sfhe::twiddles(cc.m[i].q, N, t, &cc.ninv[i], &cc.wlast[i]);
+    }
     const size_t kw = key_words(cc);
     if (cudaMalloc(&c->d_tw, tw.size() * 8) != cudaSuccess || cudaMalloc(&c->d_s, (size_t)(L + 1) * N * 8) != cudaSuccess ||
         cudaMalloc(&c->d_rlk, 2 * kw * 8) != cudaSuccess || cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess)
@@ -680,10 +723,10 @@ extern "C" sfhe_status sfhe_ckks_ctx_create(const sfhe_ckks_params* params, uint
     for (uint32_t j = 0; j < N / 2; j++, x = x * 3 % (2 * (int64_t)N)) c->slot_exp[j] = x;
     cudaError_t e = cudaSuccess;
     auto secret = [&]() -> cudaError_t {
-        CK_DISPATCH(cc.logN, {
-            cudaError_t ee = ck_allow(k_ck_secret<LG>, ck_smem<LG>());
+        CK_DISPATCH_NTT(cc, {
+            cudaError_t ee = ck_allow(k_ck_secret<LG, PM>, ck_smem<LG>());
             if (ee != cudaSuccess) return ee;
-            k_ck_secret<LG><<<L + 1, ck_nt<LG>(), ck_smem<LG>(), 0>>>(cc, c->d_s, c->d_err);
+            k_ck_secret<LG, PM><<<L + 1, ck_nt<LG>(), ck_smem<LG>(), 0>>>(cc, c->d_s, c->d_err);
             return cudaGetLastError();
         });
     };
@@ -843,10 +886,10 @@ extern "C" sfhe_status sfhe_ckks_encrypt(sfhe_ckks_ctx* c, const int64_t* polys,
     cudaError_t e;
     {
         auto launch = [&]() -> cudaError_t {
-            CK_DISPATCH(c->cc.logN, {
-                cudaError_t ee = ck_allow(k_ck_encrypt<LG>, ck_smem<LG>());
+            CK_DISPATCH_NTT(c->cc, {
+                cudaError_t ee = ck_allow(k_ck_encrypt<LG, PM>, ck_smem<LG>());
                 if (ee != cudaSuccess) return ee;
-                k_ck_encrypt<LG><<<dim3(c->cc.L, (unsigned)n), ck_nt<LG>(), ck_smem<LG>(), s>>>(
+                k_ck_encrypt<LG, PM><<<dim3(c->cc.L, (unsigned)n), ck_nt<LG>(), ck_smem<LG>(), s>>>(
                     c->cc, c->d_s, d_polys, d_coords, matrix_id, ct, c->d_err);
                 return cudaGetLastError();
             });

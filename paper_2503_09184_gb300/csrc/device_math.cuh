@@ -121,6 +121,36 @@ SFHE_DEV u64 pm_canon(i64 v, u64 q)
     r += r < 0 ? (i64)q : 0;
     return r >= (i64)q ? (u64)r - q : (u64)r;
 }
+// The same arithmetic for a prime of any n bits, 32 < n <= 54, q = 2^n - c,
+// c < 2^23 (constants split at bit n - 32): |p1| and |p0| keep their bounds, so
+// the products stay within 2^55 as above however small q is.
+SFHE_DEV int pm_bits(u64 q) { return 64 - __clzll((long long)q); }
+SFHE_DEV int pm_c_any(u64 q) { return (int)((1ULL << pm_bits(q)) - q); }
+SFHE_DEV i64 pm_mul_any(i64 a, u64 w, u64 w2, int c, int n)
+{
+    const int a0 = (int)a, a1 = (int)(a >> 32) + (int)((u32)a0 >> 31);
+    const i64 p1 = mad_wide(a1, (int)(w2 >> 32), mul_wide(a0, (int)(w >> 32)));
+    const i64 p0 = mad_wide(a1, (int)w2, mul_wide(a0, (int)w));
+    return mad_wide((int)(p1 >> 32), c, p0) + (i64)((u64)(u32)p1 << (n - 32));
+}
+// one fold of |v| < 2^62: below 2^54 in magnitude (h c < 2^29 2^23)
+SFHE_DEV i64 pm_fold_any(i64 v, int c, int n)
+{
+    return mad_wide((int)(v >> n), c, (i64)((u64)v & ((1ULL << n) - 1)));
+}
+// the same for any unsigned word: below 2^55
+SFHE_DEV i64 pm_fold_any_u(u64 v, int c, int n)
+{
+    return mad_wide((int)(u32)(v >> n), c, (i64)(v & ((1ULL << n) - 1)));
+}
+// canonical residue of |v| < 2^62: three folds leave one correction either way (n > 32)
+SFHE_DEV u64 pm_canon_any(i64 v, u64 q)
+{
+    const int n = pm_bits(q), c = pm_c_any(q);
+    i64 r = pm_fold_any(pm_fold_any(pm_fold_any(v, c, n), c, n), c, n);
+    r += r < 0 ? (i64)q : 0;
+    return r >= (i64)q ? (u64)r - q : (u64)r;
+}
 // the constant's two packed words from its canonical residue
 SFHE_DEV u64 pm_pack(u64 w, u64 q)
 {

@@ -250,28 +250,37 @@ void twiddles(uint64_t q, uint32_t N, uint64_t* out, ShoupC* ninv, ShoupC* wlast
     *wlast = shoup_of(mulm(g[1], ni, q), q);
 }
 
+static int bits_of(uint64_t q) { return 64 - __builtin_clzll(q); }
+
+bool pm_fits(uint64_t q)
+{
+    const int n = bits_of(q);
+    return n > 32 && n <= 54 && (1ULL << n) - q < (1ULL << 23);
+}
+
 static uint64_t pm_pack(uint64_t w, uint64_t q)
 {
+    const int64_t unit = (int64_t)1 << (bits_of(q) - 32);
     const int64_t s = w > q / 2 ? (int64_t)w - (int64_t)q : (int64_t)w;
-    const int64_t lo = s & ((1 << 22) - 1);  // floor remainder
-    return ((uint64_t)(uint32_t)(int32_t)((s - lo) / (1 << 22)) << 32) | (uint64_t)lo;
+    const int64_t lo = s & (unit - 1);  // floor remainder
+    return ((uint64_t)(uint32_t)(int32_t)((s - lo) / unit) << 32) | (uint64_t)lo;
 }
 
 PmC pm_of(uint64_t w, uint64_t q)
 {
     PmC c;
     c.w = pm_pack(w, q);
-    c.w2 = pm_pack(mulm(w, 1ULL << 32, q), q);
+    c.w2 = pm_pack(mulm(w, (1ULL << 32) % q, q), q);
     return c;
 }
 
-void twiddles_pm(uint64_t q, uint32_t N, uint64_t* out, PmC* ninv, PmC* wlast)
+void twiddles_pm(uint64_t q, uint32_t N, uint32_t R, uint64_t* out, PmC* ninv, PmC* wlast)
 {
     std::vector<uint64_t> f, g;
     root_tables(q, N, f, g);
-    const uint32_t nt = N / 16;  // threads of the transform
+    const uint32_t nt = N / R;  // threads of the transform
     for (uint32_t k = 0; k < N; ++k) {
-        // levels of the pass on runs of 16 elements: lane-interleaved
+        // levels of the pass on runs of R elements: lane-interleaved
         uint32_t at = k;
         if (k >= nt) {
             uint32_t base = nt;
@@ -393,7 +402,7 @@ bool fill_constants(RnsConsts& rc)
     const int L = rc.L, K = rc.K;
     for (int i = 0; i < L; ++i) {
         // pm_mul's range analysis: q = 2^54 - c, c < 2^23
-        if (rc.m[i].q >> 54 || (1ULL << 54) - rc.m[i].q >= (1ULL << 23)) return false;
+        if (bits_of(rc.m[i].q) != 54 || !pm_fits(rc.m[i].q)) return false;
         rc.ninv[i] = shoup_of(invm(rc.N, rc.m[i].q), rc.m[i].q);
     }
     const uint64_t t = rc.t;

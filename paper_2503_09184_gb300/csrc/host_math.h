@@ -28,7 +28,10 @@ void twiddles(uint64_t q, uint32_t N, uint64_t* out4N, ShoupC* ninv, ShoupC* wla
 // The same for q = 2^54 - c in pm_mul's form: [2][N] pairs (PmC), of psi_rev
 // and of ipsi_rev, the levels of the pass on runs of 16 elements
 // lane-interleaved (NttT::tw_pair).
-void twiddles_pm(uint64_t q, uint32_t N, uint64_t* out4N, PmC* ninv, PmC* wlast);
+// (runs of R elements per thread; a prime of any 33 to 54 bits.)
+void twiddles_pm(uint64_t q, uint32_t N, uint32_t R, uint64_t* out4N, PmC* ninv, PmC* wlast);
+// q = 2^n - c, 32 < n <= 54, c < 2^23: what the products' range analysis takes
+bool pm_fits(uint64_t q);
 PmC pm_of(uint64_t w, uint64_t q);
 void twiddles32(uint32_t b, uint32_t N, uint32_t* out4N, Shoup32* ninv, Shoup32* wlast);
 // Fills every base-conversion constant of rc from its primes (rc.m[].q,

@@ -28,7 +28,7 @@
 //   Arith54, primes q = 2^54 - c in signed 64-bit words (pm_mul): forward
 //     accepts |x| < 2^58 and adds less than 2^55 per stage (no reductions);
 //     inverse doubles the sums' range at every stage and folds them once per
-//     FOLD_STAGES stages; outputs are reduced by canon().
+//     FOLD_STAGES stages; outputs are reduced by pm_canon.
 //   Arith32, primes 2^29 < b < 2^30 in 32-bit words: forward keeps [0, 4b)
 //     (input below 4b), inverse keeps [0, 2b).
 #pragma once
@@ -61,19 +61,28 @@ struct Arith64 {
     }
 };
 
-struct Arith54 {
+template <bool ANY>  // ANY: a prime of any 33 to 54 bits, else 54 bits
+struct ArithPm {
     using W = u64;
-    // inverse: canonical inputs are below 2^54; after s stages without a fold
-    // the sums are below 2^(54+s), the differences fed to pm_mul below
+    // inverse: inputs are below 2^54; after s stages without a fold the sums
+    // are below 2^(54+s), the differences fed to the product below
     // 2^(54+s): eight stages stay within its range
     static constexpr int FOLD_STAGES = 8;
     static constexpr bool PAIRS = true;  // twiddle layout: see tw_pair
-    SFHE_DEV static W fold(W x, W q) { return (W)pm_fold((i64)x, pm_c(q)); }
-    SFHE_DEV static W canon(W x, W q) { return pm_canon((i64)x, q); }
+    SFHE_DEV static W mul(W a, W w, W w2, W q)
+    {
+        if constexpr (ANY) return (W)pm_mul_any((i64)a, w, w2, pm_c_any(q), pm_bits(q));
+        else return (W)pm_mul((i64)a, w, w2, pm_c(q));
+    }
+    SFHE_DEV static W fold(W x, W q)
+    {
+        if constexpr (ANY) return (W)pm_fold_any((i64)x, pm_c_any(q), pm_bits(q));
+        else return (W)pm_fold((i64)x, pm_c(q));
+    }
     template <bool LEAN>
     SFHE_DEV static void fwd(W& X, W& Y, W w, W w2, W q)
     {
-        const W T = (W)pm_mul((i64)Y, w, w2, pm_c(q));
+        const W T = mul(Y, w, w2, q);
         Y = X - T;
         X = X + T;
     }
@@ -82,15 +91,16 @@ struct Arith54 {
     {
         const W s = X + Y, d = X - Y;
         X = s;
-        Y = (W)pm_mul((i64)d, w, w2, pm_c(q));
+        Y = mul(d, w, w2, q);
     }
     SFHE_DEV static void inv_last(W& X, W& Y, W ni, W ni2, W wl, W wl2, W q)
     {
         const W s = X + Y, d = X - Y;
-        X = (W)pm_mul((i64)s, ni, ni2, pm_c(q));
-        Y = (W)pm_mul((i64)d, wl, wl2, pm_c(q));
+        X = mul(s, ni, ni2, q);
+        Y = mul(d, wl, wl2, q);
     }
 };
+using Arith54 = ArithPm<false>;
 
 struct Arith32 {
     using W = u32;
