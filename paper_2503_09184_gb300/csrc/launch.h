@@ -83,7 +83,6 @@ cudaError_t launch_encrypt_poly(const RnsConsts& rc, const u64* s_ntt, const lon
 // w: n L N words of scratch; out: n N message digits in [0, t) (device)
 cudaError_t launch_decrypt_poly(const RnsConsts& rc, const u64* s_ntt, const u64* ct, long long n, u64* w,
                                 long long* out, cudaStream_t s);
-cudaError_t launch_galois_apply(const RnsConsts& rc, const u64* in, long long n, u32 g, u64* out, cudaStream_t s);
 cudaError_t launch_mul_plain(const RnsConsts& rc, u64* ct, long long n, const u64* pt, cudaStream_t s);
 cudaError_t launch_add_ct(const RnsConsts& rc, u64* acc, const u64* x, long long n, cudaStream_t s);
 size_t rotate_work_words(const RnsConsts& rc);

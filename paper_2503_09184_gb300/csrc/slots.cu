@@ -173,17 +173,6 @@ __global__ void __launch_bounds__(256) k_dec_round(const __grid_constant__ RnsCo
     out[idx] = (long long)((usum + kk) % c.t);
 }
 
-// out = ct with X -> X^g applied to both polynomials (NTT form: a gather)
-template <int LOGN>
-__global__ void __launch_bounds__(256) k_galois_apply(const __grid_constant__ RnsConsts c, const u64* in, u32 g, u64* out)
-{
-    constexpr int N = 1 << LOGN;
-    const int k = blockIdx.x * 256 + threadIdx.x;
-    const size_t poly = blockIdx.y;  // n * 2L + p L + l
-    if (k >= N) return;
-    out[poly * N + k] = in[poly * N + galois_src<LOGN>(k, g)];
-}
-
 // ct[n][p][l] *= pt[l] (NTT form)
 __global__ void __launch_bounds__(256) k_mul_plain(const __grid_constant__ RnsConsts c, u64* ct, const u64* pt)
 {
@@ -245,8 +234,7 @@ __global__ void __launch_bounds__(256) k_galois_apply_b(const __grid_constant__ 
     out[blockIdx.z * out_stride + poly * N + k] = in[blockIdx.z * in_stride + poly * N + galois_src<LOGN>(k, g)];
 }
 
-// block (target limb i, source s, ciphertext z): forward NTT of d0 limb i
-// (s = 0), of d1 limb i (s = 1), of digit j = s - 2 mod q_i (s >= 2)
+// block (target limb i, digit j, ciphertext z): forward NTT of digit j mod q_i
 template <int LOGN>
 __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_ks_ntt(const __grid_constant__ RnsConsts c, const u64* D,
                                                                 size_t d_stride, u64* U, size_t u_stride)
@@ -254,61 +242,62 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_ks_ntt(const __grid_co
     using NT_ = typename NttGeom<LOGN>::T;
     constexpr int N = NT_::N;
     extern __shared__ u64 sm[];
-    const int i = blockIdx.x, s = blockIdx.y, tid = threadIdx.x, L = c.L;
+    const int i = blockIdx.x, j = blockIdx.y, tid = threadIdx.x, L = c.L;
     const Mod m = c.m[i];
-    const u64* Dz = D + blockIdx.z * d_stride;
-    const u64* src = s == 0 ? Dz + (size_t)i * N : (s == 1 ? Dz + ((size_t)L + i) * N : Dz + ((size_t)2 * L + (s - 2)) * N);
+    const u64* src = D + blockIdx.z * d_stride + (size_t)j * N;
     u64 x[NT_::R];
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) x[v] = src[NT_::fwd_in_idx(v, tid)];
     NT_::forward(x, sm, tid, c.tw + (size_t)i * 4 * N, m.q);
-    u64* dst = U + blockIdx.z * u_stride + ((size_t)s * L + i) * N;
+    u64* dst = U + blockIdx.z * u_stride + ((size_t)j * L + i) * N;
     NT_::run_to_lane(x, sm, tid);
 #pragma unroll
     for (int v = 0; v < NT_::R; v++) dst[NT_::lane_idx(v, tid)] = pm_canon((i64)x[v], m.q);
 }
 
-// out[p][i] = U[p][i] + sum_j U[2+j][i] key[j][p][i]   (p = 0: b, 1: a)
-__global__ void __launch_bounds__(256) k_ks_accum(const __grid_constant__ RnsConsts c, const u64* U, size_t u_stride,
-                                                  const u64* key, const u64* key_sh, u64* out, size_t out_stride)
+// out[p][i] = [p = 0] P[0][i] + sum_j U[j][i] key[j][p][i]   (p = 0: b, 1: a)
+__global__ void __launch_bounds__(256) k_ks_accum(const __grid_constant__ RnsConsts c, const u64* P, size_t p_stride,
+                                                  const u64* U, size_t u_stride, const u64* key, const u64* key_sh,
+                                                  u64* out, size_t out_stride)
 {
     const int N = c.N, L = c.L;
     const int k = blockIdx.x * 256 + threadIdx.x, i = blockIdx.y;
     if (k >= N) return;
     const Mod m = c.m[i];
     const u64* Uz = U + blockIdx.z * u_stride;
-    for (int p = 0; p < 2; p++) {
-        u64 acc = Uz[((size_t)p * L + i) * N + k];
-        for (int j = 0; j < L; j++) {
-            const size_t ro = (((size_t)j * 2 + p) * L + i) * N + k;
-            acc += shoup_lazy(Uz[((size_t)(2 + j) * L + i) * N + k], key[ro], key_sh[ro], m.q);
-        }
-        out[blockIdx.z * out_stride + ((size_t)p * L + i) * N + k] = barrett64(acc, m);
+    u64 s0 = P[blockIdx.z * p_stride + (size_t)i * N + k], s1 = 0;
+    for (int j = 0; j < L; j++) {
+        const u64 x = Uz[((size_t)j * L + i) * N + k];
+        const size_t rb = (((size_t)j * 2 + 0) * L + i) * N + k, ra = (((size_t)j * 2 + 1) * L + i) * N + k;
+        s0 += shoup_lazy(x, key[rb], key_sh[rb], m.q);
+        s1 += shoup_lazy(x, key[ra], key_sh[ra], m.q);
     }
+    out[blockIdx.z * out_stride + (size_t)i * N + k] = barrett64(s0, m);
+    out[blockIdx.z * out_stride + ((size_t)L + i) * N + k] = barrett64(s1, m);
 }
 
+// P = sigma_g(in) in NTT form; c0's part is added as it is, c1's goes to
+// coefficient form for its digits: L inverse and L^2 forward transforms per
+// ciphertext (20 at L = 4).  Sending both parts through the relinearisation's
+// sources took 2 L + (L + 2) L (32): chunked 16^3 at c = 8 (GB300) 9.2 -> 8.1 ms.
 template <int LOGN>
 cudaError_t rotate_batch_impl(const RnsConsts& rc, const u64* in, size_t in_stride, long long n, u32 g, const u64* key,
                               const u64* key_sh, u64* out, size_t out_stride, u64* work, cudaStream_t s)
 {
     const size_t LN = (size_t)rc.L * rc.N;
-    const size_t pw = 2 * LN, dw = 3 * LN, uw = (size_t)(rc.L + 2) * LN;
+    const size_t pw = 2 * LN, dw = LN, uw = (size_t)rc.L * LN;
     u64* P = work;
     u64* D = P + (size_t)n * pw;
     u64* U = D + (size_t)n * dw;
     const unsigned bx = (unsigned)((rc.N + 255) / 256);
     k_galois_apply_b<LOGN><<<dim3(bx, 2 * rc.L, (unsigned)n), 256, 0, s>>>(rc, in, in_stride, g, P, pw);
     cudaError_t e = cudaGetLastError();
-    // d0 = sigma_g(c0), d1 = 0, d2 = sigma_g(c1), coefficient form (canonical)
-    if (e == cudaSuccess) e = launch_ntt(rc, true, P, pw, 0, D, dw, 0, 0, rc.L, n, s);
-    if (e == cudaSuccess) e = launch_ntt(rc, true, P, pw, rc.L, D, dw, 2 * rc.L, 0, rc.L, n, s);
-    if (e == cudaSuccess) e = cudaMemset2DAsync(D + LN, dw * 8, 0, LN * 8, (size_t)n, s);
+    if (e == cudaSuccess) e = launch_ntt(rc, true, P, pw, rc.L, D, dw, 0, 0, rc.L, n, s);
+    if (e == cudaSuccess) e = allow_smem(k_ks_ntt<LOGN>, smem_of<LOGN>());
     if (e != cudaSuccess) return e;
-    e = allow_smem(k_ks_ntt<LOGN>, smem_of<LOGN>());
-    if (e != cudaSuccess) return e;
-    k_ks_ntt<LOGN><<<dim3(rc.L, rc.L + 2, (unsigned)n), nt_of<LOGN>(), smem_of<LOGN>(), s>>>(rc, D, dw, U, uw);
+    k_ks_ntt<LOGN><<<dim3(rc.L, rc.L, (unsigned)n), nt_of<LOGN>(), smem_of<LOGN>(), s>>>(rc, D, dw, U, uw);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_ks_accum<<<dim3(bx, rc.L, (unsigned)n), 256, 0, s>>>(rc, U, uw, key, key_sh, out, out_stride);
+    k_ks_accum<<<dim3(bx, rc.L, (unsigned)n), 256, 0, s>>>(rc, P, pw, U, uw, key, key_sh, out, out_stride);
     return cudaGetLastError();
 }
 
@@ -369,23 +358,6 @@ cudaError_t launch_decrypt_poly(const RnsConsts& rc, const u64* s_ntt, const u64
     const long long total = n * rc.N;
     k_dec_round<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(rc, w, out, total);
     return cudaGetLastError();
-}
-
-cudaError_t launch_galois_apply(const RnsConsts& rc, const u64* in, long long n, u32 g, u64* out, cudaStream_t s)
-{
-    const unsigned bx = (unsigned)((rc.N + 255) / 256);
-    const long long polys = n * 2 * rc.L;
-    for (long long p0 = 0; p0 < polys; p0 += 65535) {
-        const long long cnt = polys - p0 < 65535 ? polys - p0 : 65535;
-        SLOTS_DISPATCH_LOGN(rc.logN, {
-            k_galois_apply<LG><<<dim3(bx, (unsigned)cnt), 256, 0, s>>>(rc, in + (size_t)p0 * rc.N, g,
-                                                                        out + (size_t)p0 * rc.N);
-            break;
-        });
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 cudaError_t launch_mul_plain(const RnsConsts& rc, u64* ct, long long n, const u64* pt, cudaStream_t s)
@@ -460,34 +432,16 @@ cudaError_t launch_rotate_batch(const RnsConsts& rc, const u64* in, size_t in_st
     return cudaSuccess;
 }
 
-// Rotation of one ciphertext: P = sigma_g(in) (NTT form); its two
-// polynomials back to coefficient form give d0 = sigma_g(c0) and the digits
-// D_j = [sigma_g(c1)]_{q_j} (canonical); with d1 = 0 the relinearisation
-// kernels then form out = (d0 + sum_j D_j b_j, sum_j D_j a_j) with the
-// Galois key in place of the relinearisation key.
-// work: P [2][L][N], D [3][L][N], U [(L+2)][L][N] (uint64).
+// Rotation of one ciphertext: a batch of one.  Work per ciphertext: P
+// [2][L][N], the digits [L][N] and their transforms [L][L][N] (uint64; the
+// callers' workspaces keep room for four more rows of L N words).
 size_t rotate_work_words(const RnsConsts& rc) { return (size_t)(2 + 3 + rc.L + 2) * rc.L * rc.N; }
 
 cudaError_t launch_rotate(const RnsConsts& rc, const u64* in, u32 g, const u64* key, const u64* key_sh, u64* out,
                           u64* work, cudaStream_t s)
 {
-    const size_t LN = (size_t)rc.L * rc.N;
-    u64* P = work;
-    u64* D = P + 2 * LN;
-    u64* U = D + 3 * LN;
-    cudaError_t e = launch_galois_apply(rc, in, 1, g, P, s);
-    if (e == cudaSuccess) e = launch_ntt(rc, true, P, LN, 0, D, LN, 0, 0, rc.L, 1, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D + LN, 0, LN * 8, s);
-    if (e == cudaSuccess) e = launch_ntt(rc, true, P + LN, LN, 0, D + 2 * LN, LN, 0, 0, rc.L, 1, s);
-    if (e != cudaSuccess) return e;
-    SLOTS_DISPATCH_LOGN(rc.logN, {
-        if ((e = allow_smem(k_ks_ntt<LG>, smem_of<LG>())) != cudaSuccess) return e;
-        k_ks_ntt<LG><<<dim3(rc.L, rc.L + 2, 1), nt_of<LG>(), smem_of<LG>(), s>>>(rc, D, 0, U, 0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        break;
-    });
-    k_ks_accum<<<dim3((unsigned)((rc.N + 255) / 256), rc.L, 1), 256, 0, s>>>(rc, U, 0, key, key_sh, out, 0);
-    return cudaGetLastError();
+    const size_t ctw = (size_t)2 * rc.L * rc.N;
+    return launch_rotate_batch(rc, in, ctw, 1, g, key, key_sh, out, ctw, work, 1, s);
 }
 
 }  // namespace sfhe
