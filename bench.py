@@ -868,7 +868,8 @@ def e2e_host(args, api, S, torch, ctx, slot0, products, world) -> dict:
 # launch; valid only for the kernel sources it was taken on (their hash).
 KERNEL_SOURCES = ("kernels.cuh", "ntt.cuh", "device_math.cuh", "rns.h", "launch.h", "persistent_impl.cuh",
                   "persistent_12.cu", "persistent_13.cu", "persistent_14.cu", "persistent_tuned_12.cu",
-                  "persistent_tuned_13.cu", "persistent_tuned_13b.cu", "persistent_tuned_14.cu")
+                  "persistent_tuned_13.cu", "persistent_tuned_13b.cu", "persistent_tuned_14.cu", "round_mma.cuh",
+                  "round_shape.h")
 TRAFFIC = {  # (source hash, workload) -> (bytes per launch, profile summary)
     ("a6654f27039fa051", "sweep-64x64x64-s0.5"): (715.07e9, "profiles/matmul_persistent_sweep64x64x64_s0.5_dram.md"),
     ("a6654f27039fa051", "sweep-64x64x64-s0.5-lazy"): (170.46e9,

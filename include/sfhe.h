@@ -145,7 +145,7 @@ typedef struct {
 /* Parameters and keys.  Selects the primes, builds the NTT and base
  * conversion tables, and runs key generation on the current device from
  * `seed` (secret and relinearisation key never leave the device unless
- * exported).  Synchronous.  The key and its Shoup companions share one
+ * exported).  Synchronous.  The key and its prepared form share one
  * allocation, over which every persistent launch carries a persisting-L2
  * access-policy window: the context raises its persisting-L2 limit (a limit
  * of this process's CUDA context, gone with it) up to the key's size.  The
@@ -593,7 +593,8 @@ sfhe_status sfhe_selftest_wait_bound(void* work, uint32_t tries, uint32_t limit_
 /* Tile tuning of the per-product persistent kernel.  Where a ring has
  * several tiles (stage-S tiles of the exact scale-and-round: how many
  * coefficients a thread rounds at a time and how many output primes it
- * reconstructs per pass; and code forms of the tensor's inverse NTT: lean
+ * reconstructs per pass, or, at L = 8, when the sums are loaded around its
+ * matrix product; and code forms of the tensor's inverse NTT: lean
  * exchange addresses and reductions, a warp-shuffle stage; N = 4096 with
  * L = 2 and N = 16384 with L = 8 have three tiles, N = 8192 with L = 4
  * five), the first per-product persistent plan of a context times every

@@ -958,7 +958,7 @@ sfhe_status launch_plan(sfhe_plan* P, cudaStream_t s)
             CUDA_TRY(launch_tensor_intt(rc, a, b, P->d_T, s));
             CUDA_TRY(launch_scale_round(rc, P->d_T, P->d_D, s));
             CUDA_TRY(launch_relin_ntt(rc, P->d_D, P->d_U, s));
-            CUDA_TRY(launch_relin_accum(rc, P->d_U, c->d_rlk_pm, Cout, s));
+            CUDA_TRY(launch_relin_accum(rc, P->d_U, c->d_rlk_pm, Cout, true, s));
         }
     }
     return SFHE_OK;
@@ -1341,11 +1341,10 @@ extern "C" sfhe_status sfhe_ct_mul_relin(sfhe_ctx* c, const uint32_t* a_ext, con
     u32* T = (u32*)work;
     u64* D = (u64*)((char*)work + tw);
     u64* U = D + 3 * L * N;
-    CUDA_TRY(cudaMemsetAsync(out, 0, 2 * L * N * 8, s));
     CUDA_TRY(launch_tensor_intt(c->rc, a_ext, b_ext, T, s));
     CUDA_TRY(launch_scale_round(c->rc, T, D, s));
     CUDA_TRY(launch_relin_ntt(c->rc, D, U, s));
-    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, s));
+    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, false, s));
     return SFHE_OK;
 }
 
@@ -1378,11 +1377,10 @@ extern "C" sfhe_status sfhe_ct_mul_relin_static(sfhe_ctx* c, const uint32_t* a_e
     u32* T = (u32*)base;
     u64* D = (u64*)((char*)base + tw);
     u64* U = D + 3 * L * N;
-    CUDA_TRY(cudaMemsetAsync(out, 0, 2 * L * N * 8, s));
     CUDA_TRY(launch_tensor_intt(c->rc, a_ext, b_ext, T, s));
     CUDA_TRY(launch_scale_round(c->rc, T, D, s));
     CUDA_TRY(launch_relin_ntt(c->rc, D, U, s));
-    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, s));
+    CUDA_TRY(launch_relin_accum(c->rc, U, c->d_rlk_pm, out, false, s));
     return SFHE_OK;
 }
 

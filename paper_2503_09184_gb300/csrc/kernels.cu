@@ -226,9 +226,10 @@ cudaError_t launch_relin_ntt(const RnsConsts& rc, const u64* D, u64* U, cudaStre
     });
 }
 
-cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, cudaStream_t s)
+cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, bool add,
+                               cudaStream_t s)
 {
-    k_relin_accum<<<dim3((rc.N + 255) / 256, rc.L), 256, 0, s>>>(rc, U, rlk_pm, C);
+    k_relin_accum<<<dim3((rc.N + 255) / 256, rc.L), 256, 0, s>>>(rc, U, rlk_pm, C, add ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -616,10 +616,10 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T::NT) k_relin_ntt(const __grid
 }
 
 #ifdef SFHE_KERNELS_TU
-// C[p][i] += U[p][i] + sum_j U[2+j][i] rlk[j][p][i]   (p = 0: b, 1: a); U and
+// C[p][i] (+)= U[p][i] + sum_j U[2+j][i] rlk[j][p][i]   (p = 0: b, 1: a; add: into C, else stored); U and
 // the key lane-interleaved, R = 16 words per thread of the transform
 __global__ void __launch_bounds__(256) k_relin_accum(const __grid_constant__ RnsConsts c, const u64* U, const u64* rlk_pm,
-                                                     u64* C)
+                                                     u64* C, int add)
 {
     const int N = c.N, L = c.L;
     const int k = blockIdx.x * 256 + threadIdx.x, i = blockIdx.y;
@@ -634,7 +634,8 @@ __global__ void __launch_bounds__(256) k_relin_accum(const __grid_constant__ Rns
             acc += pm_mul((i64)U[((size_t)(2 + j) * L + i) * N + k], w.x, w.y, pc);
         }
         u64* cp = C + ((size_t)p * L + i) * N + e;
-        *cp = add_mod(*cp, pm_canon(acc, m.q), m.q);
+        const u64 w = pm_canon(acc, m.q);
+        *cp = add ? add_mod(*cp, w, m.q) : w;
     }
 }
 

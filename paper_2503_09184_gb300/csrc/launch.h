@@ -35,7 +35,8 @@ cudaError_t launch_lift_extend(const RnsConsts& rc, const u64* in, u32* out, lon
 cudaError_t launch_tensor_intt(const RnsConsts& rc, const u32* a, const u32* b, u32* T, cudaStream_t s);
 cudaError_t launch_scale_round(const RnsConsts& rc, const u32* T, u64* D, cudaStream_t s);
 cudaError_t launch_relin_ntt(const RnsConsts& rc, const u64* D, u64* U, cudaStream_t s);
-cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, cudaStream_t s);
+// add: into C, else C is only written
+cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk_pm, u64* C, bool add, cudaStream_t s);
 // fused persistent path (persistent_<logN>.cu).  One launch: the work list,
 // the key, the per-CTA scratch, the grid, the mode, the tile variant and a
 // persisting-L2 access-policy window (over the relinearisation key;
