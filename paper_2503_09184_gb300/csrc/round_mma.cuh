@@ -21,7 +21,8 @@
 // spends about 10 (L + 1): as a contraction of length 4 K with 6 L + 7 columns
 // its products cost the tensor pipe a few per cent of the stage.  At L = 8,
 // N = 16384 the stage was a third of the kernel: two 32 x 64 x 16 matmuls at
-// 60% zeros 267 -> 234 ms (GB300).  At L <= 4 (K <= 16) the two forms issue about as many
+// 60% zeros 267 -> 241 ms (GB300; 0.92 -> 0.83 of one earlier build timed
+// beside both).  At L <= 4 (K <= 16) the two forms issue about as many
 // instructions, 450 per coefficient and warp, and the stage waits for its
 // residues and sums instead (2.3 MB of scratch per CTA, more than the CTAs'
 // share of L2): measured with byte subnormals, bulk-copied residues and
