@@ -38,11 +38,17 @@
 #include "round_shape.h"
 
 // ------------------------------------------------------ tensor memory -----
+// The tcgen05 instructions with .sync.aligned are the warp's: PTX leaves them
+// undefined unless all 32 lanes execute them together, which independent
+// thread scheduling does not give after a branch or a spin that lanes leave
+// at different times.  So every sequence of them starts with a __syncwarp()
+// (tmem_alloc, tmem_dealloc, RoundMma::store_row, RoundMma::load_row).
 // one warp; COLS a power of two, at least 32 (an immediate: with a register
 // the occupancy calculation assumes all 512 columns)
 template <int COLS>
 SFHE_DEV void tmem_alloc(u32* slot)
 {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "n"(COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -50,6 +56,7 @@ SFHE_DEV void tmem_alloc(u32* slot)
 template <int COLS>
 SFHE_DEV void tmem_dealloc(u32 base)  // the same warp
 {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "n"(COLS) : "memory");
 }
 SFHE_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -101,12 +108,14 @@ struct RoundMma {
         asm("sub.f16x2 %0, %0, %1;" : "+r"(w0) : "r"(0x64806480u));
         asm("sub.f16x2 %0, %0, %1;" : "+r"(w1) : "r"(0x64806480u));
     }
-    // the coefficient's row: residues at src[k * stride] into the columns at `a`
+    // the coefficient's row: residues at src[k * stride] into the columns at
+    // `a`; by whole warps
     SFHE_DEV static void store_row(const u32* __restrict__ src, size_t stride, u32 a)
     {
         u32 x[K];
 #pragma unroll
         for (int k = 0; k < K; k++) x[k] = src[(size_t)k * stride];
+        __syncwarp();
 #pragma unroll
         for (int k0 = 0; k0 < KC / 4; k0 += 4) {
             u32 w[8];
@@ -143,11 +152,12 @@ struct RoundMma {
     // prime i, congruent and below 2^55.3; returns false when F is too close
     // to a half-integer to round (bits 27..53 of its fraction all equal after
     // adding a half; its error is below 2^15 units of 2^-54), and r is then
-    // not valid.
+    // not valid.  By whole warps.
     template <int NP>  // NP = L
     SFHE_DEV static bool load_row(u32 d, const RnsConsts& c, u64 (&out)[NP])
     {
         u32 r[32];
+        __syncwarp();
 #pragma unroll
         for (int q = 0; q < 4; q++) tmem_ld8(reinterpret_cast<u32(&)[8]>(r[8 * q]), d + 8 * q);
         tmem_wait_ld();

@@ -1,0 +1,49 @@
+"""How the sources use the warp-collective tensor-memory instructions, read as
+text: the rules that a run cannot show to be kept, since a broken one goes
+wrong only where the compiler or the scheduler makes it."""
+from __future__ import annotations
+
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_09184_gb300", "csrc")
+
+
+def _read(name):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+
+
+def _functions(text):
+    """{name: body} of the brace-delimited functions (device ones, members included)"""
+    out = {}
+    for m in re.finditer(r"SFHE_DEV\s+(?:static\s+)?\w+\s+(\w+)\(", text):
+        i = text.index("{", m.end())
+        depth, j = 1, i + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[j], 0)
+            j += 1
+        out[m.group(1)] = text[i:j]
+    return out
+
+
+def test_collective_instructions_follow_a_warp_barrier():
+    """PTX leaves a .sync.aligned instruction undefined in a diverged warp:
+    each sequence of them starts with __syncwarp()"""
+    fns = _functions(_read("round_mma.cuh"))
+    collective = {n for n, body in fns.items() if ".sync.aligned" in body}
+    assert {"tmem_alloc", "tmem_dealloc", "tmem_st8", "tmem_ld8", "tmem_wait_st", "tmem_wait_ld"} <= collective
+    guarded = set()
+    for name, body in fns.items():
+        first = min([m.start() for c in collective - {name} for m in re.finditer(r"\b%s\b" % c, body)] +
+                    [m.start() for m in re.finditer(r"\.sync\.aligned", body)], default=None)
+        if first is not None and "__syncwarp();" in body[:first]:
+            guarded.add(name)
+    assert {"tmem_alloc", "tmem_dealloc", "store_row", "load_row"} <= guarded
+    # the unguarded ones are called from the guarded ones only
+    for name in collective - guarded:
+        for other, body in fns.items():
+            if other != name and re.search(r"\b%s\b" % name, body):
+                assert other in guarded, (name, other)
+        for f in os.listdir(CSRC):
+            if f.endswith((".cu", ".cuh")) and f != "round_mma.cuh":
+                assert not re.search(r"\b%s\b" % name, _read(f)), (name, f)
