@@ -62,7 +62,16 @@ SFHE_DEV void tmem_dealloc(u32 base)  // the same warp
 SFHE_DEV void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 SFHE_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 SFHE_DEV void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-SFHE_DEV void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for the warp's loads into w.  The registers hold the columns only
+// behind the wait, which has no operands of its own: the empty statements make
+// every use of w depend on it.
+template <int NR>
+SFHE_DEV void tmem_wait_ld(u32 (&w)[NR])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < NR; i++) asm volatile("" : "+r"(w[i]));
+}
 // eight columns of the calling warp's lanes
 SFHE_DEV void tmem_st8(u32 addr, const u32* w)
 {
@@ -160,7 +169,7 @@ struct RoundMma {
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 4; q++) tmem_ld8(reinterpret_cast<u32(&)[8]>(r[8 * q]), d + 8 * q);
-        tmem_wait_ld();
+        tmem_wait_ld(r);
         const u32 v = (r[0] + c.mm_vc) >> 16;
         // F + 2^20 (the offset keeps it positive), in units of 2^-54: g0 + 2^27 g1
         const i64 g0 = mad_wide((int)v, c.mm_rb0n, (i64)join(c.mm_g0, r[1], r[2], r[3], c));
@@ -173,7 +182,7 @@ struct RoundMma {
             if (i == 4) {
 #pragma unroll
                 for (int q = 0; q < (NC > 32 ? 3 : 0); q++) tmem_ld8(reinterpret_cast<u32(&)[8]>(r[8 * q]), d + 32 + 8 * q);
-                tmem_wait_ld();
+                tmem_wait_ld(r);
             }
             constexpr int COL[8] = {7, 13, 19, 25, 0, 6, 12, 18};  // round_mma_col(i) mod 32
             const int o = COL[i];

@@ -47,3 +47,17 @@ def test_collective_instructions_follow_a_warp_barrier():
         for f in os.listdir(CSRC):
             if f.endswith((".cu", ".cuh")) and f != "round_mma.cuh":
                 assert not re.search(r"\b%s\b" % name, _read(f)), (name, f)
+
+
+def test_loaded_registers_depend_on_the_wait():
+    """the compiler may move a use of a loaded register above a wait that does
+    not name it: the wait takes the registers, and every load has one before
+    the first use"""
+    fns = _functions(_read("round_mma.cuh"))
+    wait = fns["tmem_wait_ld"]
+    assert re.search(r'asm volatile\("" : "\+r"\(w\[i\]\)\)', wait[wait.index("wait::ld"):])
+    body = fns["load_row"]
+    loads = [m.end() for m in re.finditer(r"tmem_ld8\(reinterpret_cast<u32\(&\)\[8\]>\(r\[8 \* q\]\), d[^;]*;", body)]
+    assert len(loads) == len(re.findall("tmem_ld8", body)) == 2
+    for at in loads:
+        assert body[at:].lstrip().startswith("tmem_wait_ld(r);")
