@@ -899,7 +899,13 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
         };
         // The same on the tensor cores: d0 and d1 stay below 2^55.3.  The right
         // operand is copied into the idle exchange buffers.  False (in some
-        // threads) if a matrix product did not complete within the wait bound.
+        // threads) if a matrix product did not complete within the wait bound:
+        // a thread whose wait ran out waits no more and issues no further
+        // product (its sums are not valid, and the caller leaves), and behind
+        // the loop it gives the one in flight a second bounded wait, so that
+        // the tensor memory is not given back under it.  (Leaving the loop
+        // there, by a vote of the warp, took 1.7% at N = 16384: 171.5 against
+        // 168.7 ms for 32 x 64 x 16, GB300.)
         auto stage_s_mma = [&](int pr) -> bool {
             const bool fold = pr != 0 && pr % 255 == 0;  // sums below 2^54.1 + 255 2^55.3 < 2^64
             const int wg = tid >> 7, row = tid & 127;
@@ -923,7 +929,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                 if ((row & 31) == 0) mbar_arrive(&row_bar[wg]);
                 if (row < 32) {
                     if (alive) alive = mbar_wait(&row_bar[wg], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
-                    if (row == 0) {
+                    if (row == 0 && alive) {
                         tc_fence_after();
                         RM::issue(d, a, smem_addr(smb));
                         mma_commit(&mma_bar[wg]);
@@ -936,7 +942,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
                 };
                 if constexpr (TL::EARLY) load_prev();
                 if (alive) alive = mbar_wait(&mma_bar[wg], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
-                mma_phase ^= 1u;
+                if (alive) mma_phase ^= 1u;
                 tc_fence_after();
                 const bool ok = RM::load_row(d + lane, c, w);
                 tc_fence_before();
@@ -953,6 +959,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
 #pragma unroll
                 for (int i = 0; i < L; i++) sum[(size_t)i * N] = prev[i] + w[i];
             }
+            if (!alive) mbar_wait(&mma_bar[wg], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS);
             return alive;
         };
         // stage S and the barrier behind it; false (in every thread) if a wait ran out

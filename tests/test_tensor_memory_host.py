@@ -61,3 +61,21 @@ def test_loaded_registers_depend_on_the_wait():
     assert len(loads) == len(re.findall("tmem_ld8", body)) == 2
     for at in loads:
         assert body[at:].lstrip().startswith("tmem_wait_ld(r);")
+
+
+def test_a_matrix_product_that_runs_out_of_time_is_the_last():
+    """stage S: a thread whose wait ran out issues no further product, keeps
+    the phase it waited for, and waits once more (bounded) before the kernel
+    gives its tensor memory back"""
+    text = _read("kernels.cuh")
+    i = text.index("auto stage_s_mma")
+    body = text[i:text.index("auto stage_s =", i)]
+    loop, end = body.split("return alive;")[0].rsplit("sum[(size_t)i * N] = prev[i] + w[i];", 1)
+    rows = loop.index("alive = mbar_wait(&row_bar[wg]")
+    issue = loop.index("RM::issue")
+    guard = loop.index("if (row == 0 && alive)")
+    assert rows < guard < issue and loop.count("RM::issue") == 1
+    done = loop.index("if (alive) alive = mbar_wait(&mma_bar[wg]")
+    assert issue < done < loop.index("if (alive) mma_phase ^= 1u;") < loop.index("RM::load_row")
+    assert loop.count("mma_phase ^=") == 1
+    assert re.search(r"if \(!alive\) mbar_wait\(&mma_bar\[wg\], mma_phase, SFHE_WAIT_TRIES, SFHE_WAIT_NS\);", end)
