@@ -701,28 +701,175 @@ sfhe_status build(const sfhe_ctx* c, int32_t n, const sfhe_matrix_view* A, const
 // leaves SMs idle, and one with a few times as many entries as CTAs ends on an
 // uneven last round.  Below 8 entries per CTA the products of an entry may
 // therefore be shared out over several units of at most u products; the last
-// unit to finish adds the sums up and relinearises.  u is the one whose
-// longest-first schedule is estimated shortest, in units of a product: an
-// entry's relinearisation counts 0.6 (N = 8192, L = 4: 1.17 us per entry
-// against 1.89 us per product, full chip) and a part 0.15 (its sums are
-// written and read once more).  In the grouped mode a unit holds whole rounding groups.
-// Measured (GB300): tiny 8^3 replay 502 -> 303 us, 13 x 29 x 7 one-shot 4.07 ->
-// 2.54 ms.  More than 2 units per CTA are not made (the slots' memory).
-const double kRelinCost = 0.6, kPartCost = 0.15;
+// unit to finish adds the sums up and relinearises.  u is the one whose launch
+// is estimated shortest, by playing the launch through (launch_length) with
+// the costs of unit_costs.  In the grouped mode a unit holds whole rounding
+// groups.  More than 2 units per CTA are not made (the slots' memory).
+//
+// Costs in units of a product, from launches over 1 to 1188 entries of 2 to
+// 128 products, shared out and whole, on six rings and in both modes (GB300):
+//  - a relinearisation is L (L + 2) transforms of 64-bit words against a
+//    product's 3 K of 32-bit words: measured 0.7 (L = 2), 0.85 (3), 1.0 (4)
+//    and 1.45 to 1.65 (8) of a product;
+//  - a rounding group costs 0.85, each of its products 0.15 (N = 8192, L = 4:
+//    229 and 34 us against 264 for a product rounded by itself);
+//  - a unit that shares an entry 0.1 more, and the last one of an entry reads
+//    its slots, bound by latency: per slot 0.1 (one entry) to 0.3 (48 or more at
+//    once) with 512 threads, twice that with 256, 0.15 where a second CTA on the
+//    SM hides it;
+//  - two CTAs on an SM take 1.75 times as long as one alone.
+// The estimated gains lie within 4% (one standard deviation) of the measured
+// ones, 10% where two CTAs share an SM.  One cost of 0.6 for every
+// relinearisation, without playing the launch through, shared out entries of 2
+// to 9 products that ran 1.1 to 1.4 times as long for it.
+struct UnitCosts {
+    int group, sms, per_sm, threads;
+    double relin;
+    double work(int count) const
+    {
+        return 0.85 * ((count + group - 1) / group) + 0.15 * count;
+    }
+    double slot(int shared) const  // entries shared out
+    {
+        if (per_sm > 1) return 0.15;
+        return 512.0 / threads * (0.1 + 0.2 * std::min(1.0, shared / 48.0));
+    }
+    double slowdown(int ctas) const { return 1 + 0.75 * (ctas - 1); }
+};
+const double kPartCost = 0.1;
 
-double schedule_length(const std::vector<double>& cost, int grid)
+UnitCosts unit_costs(const sfhe_ctx* c, uint32_t flags)
 {
-    // longest first onto the least loaded CTA
-    std::priority_queue<double, std::vector<double>, std::greater<double>> load;
-    double end = 0;
-    for (double x : cost) {
-        double t = x;
-        if ((int)load.size() >= grid) {
-            t += load.top();
-            load.pop();
+    UnitCosts k;
+    k.group = (flags & SFHE_EXEC_LAZY) ? c->rc.lazy_group : 1;
+    k.sms = c->num_sms;
+    k.per_sm = persistent_ctas_per_sm(c->rc);
+    k.threads = c->rc.N / ext_interleave(c->rc.logN);
+    k.relin = 0.3 + 1.45 * c->rc.L * (c->rc.L + 2) / (3.0 * c->rc.K);
+    return k;
+}
+
+// the entries in units of at most u products, longest first
+std::vector<Entry> units_of(const std::vector<Entry>& entries, int u)
+{
+    std::vector<Entry> units;
+    int slots = 0;
+    for (const Entry& e : entries) {
+        const int parts = e.count <= u ? 1 : (e.count + u - 1) / u, first_slot = parts > 1 ? slots : 0;
+        for (int p = 0; p < parts; p++) {
+            Entry x = e;
+            x.first = e.first + p * u;
+            x.count = std::min(u, e.count - p * u);
+            x.parts = parts;
+            x.first_slot = first_slot;
+            x.slot = parts > 1 ? first_slot + p : 0;
+            units.push_back(x);
         }
-        load.push(t);
-        end = std::max(end, t);
+        if (parts > 1) slots += parts;
+    }
+    std::stable_sort(units.begin(), units.end(), [](const Entry& a, const Entry& b) { return a.count > b.count; });
+    return units;
+}
+
+// The launch played through: every CTA takes the next unit when it is free,
+// the one that finishes an entry's last unit goes on to its relinearisation,
+// and the CTAs of an SM slow each other down.  Returns early, with a longer
+// time than `limit`, once it is past it.  (45 us on the host for 91 entries
+// in 168 units.)
+double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& k, double limit)
+{
+    struct Unit {
+        int count, entry, parts;
+    };
+    std::vector<Unit> units;
+    int shared = 0;
+    for (size_t e = 0; e < entries.size(); e++) {
+        const int parts = entries[e].count <= u ? 1 : (entries[e].count + u - 1) / u;
+        for (int p = 0; p < parts; p++) units.push_back(Unit{std::min(u, entries[e].count - p * u), (int)e, parts});
+        shared += parts > 1;
+    }
+    if (shared)  // the entries come longest first
+        std::stable_sort(units.begin(), units.end(), [](const Unit& a, const Unit& b) { return a.count > b.count; });
+    struct Cta {
+        double left;  // of its unit, in time alone on the SM
+        int unit;     // -1: none
+        bool last;    // nothing follows (a whole entry's work includes its relinearisation)
+    };
+    struct Event {  // an SM's next change
+        double t;
+        int order, sm;  // ties in the order of their making: units go to idle SMs first
+        bool operator>(const Event& o) const { return t != o.t ? t > o.t : order > o.order; }
+    };
+    std::vector<Cta> ctas((size_t)k.sms * k.per_sm, Cta{0, -1, false});
+    std::vector<double> at(k.sms, 0);
+    std::vector<int> busy(k.sms, 0), finished(entries.size(), 0);
+    std::vector<Event> heap;
+    heap.reserve(k.sms);
+    size_t next = 0;
+    int order = 0;
+    double end = 0;
+    const double slot = k.slot(shared);
+    auto take = [&](Cta& x) {
+        x.unit = -1;
+        if (next == units.size()) return;
+        x.unit = (int)next++;
+        const Unit& u = units[x.unit];
+        x.left = k.work(u.count);
+        x.last = u.parts == 1;
+        if (u.parts > 1) x.left += kPartCost;
+        else if (u.count) x.left += k.relin;
+    };
+    // the SM's next event; false: it is idle for good
+    auto event = [&](int sm, Event& ev) {
+        double least = 0;
+        busy[sm] = 0;
+        for (int j = 0; j < k.per_sm; j++) {
+            const Cta& x = ctas[(size_t)j * k.sms + sm];
+            if (x.unit < 0) continue;
+            busy[sm]++;
+            if (busy[sm] == 1 || x.left < least) least = x.left;
+        }
+        ev = Event{at[sm] + std::max(0.0, least) * k.slowdown(busy[sm]), order++, sm};
+        return busy[sm] > 0;
+    };
+    for (Cta& x : ctas) take(x);  // one CTA on every SM first
+    for (int sm = 0; sm < k.sms; sm++) {
+        Event ev;
+        if (event(sm, ev)) heap.push_back(ev);
+    }
+    std::make_heap(heap.begin(), heap.end(), std::greater<Event>());
+    while (!heap.empty() && end <= limit) {
+        const Event ev = heap[0];
+        Cta* done = nullptr;
+        for (int j = 0; j < k.per_sm; j++) {
+            Cta& x = ctas[(size_t)j * k.sms + ev.sm];
+            if (x.unit < 0) continue;
+            x.left -= (ev.t - at[ev.sm]) / k.slowdown(busy[ev.sm]);
+            if (!done || x.left < done->left) done = &x;
+        }
+        at[ev.sm] = end = ev.t;
+        const Unit& u = units[done->unit];
+        if (!done->last && ++finished[u.entry] == u.parts) {
+            done->left = k.relin + u.parts * slot;
+            done->last = true;
+        } else {
+            take(*done);
+        }
+        Event x;
+        if (!event(ev.sm, x)) {
+            std::pop_heap(heap.begin(), heap.end(), std::greater<Event>());
+            heap.pop_back();
+            continue;
+        }
+        // the SM's new event replaces its old one at the root
+        size_t i = 0;
+        for (size_t c = 1; c < heap.size(); c = 2 * i + 1) {
+            if (c + 1 < heap.size() && heap[c] > heap[c + 1]) c++;
+            if (!(x > heap[c])) break;
+            heap[i] = heap[c];
+            i = c;
+        }
+        heap[i] = x;
     }
     return end;
 }
@@ -734,52 +881,31 @@ void split_entries(const sfhe_ctx* c, sfhe_plan& P, uint32_t flags)
     P.last_unit.clear();
     for (Entry& e : P.entries) e.parts = 1, e.slot = e.first_slot = 0;
     if (!(flags & SFHE_EXEC_PERSISTENT) || P.entries.empty()) return;
-    const int grid = persistent_ctas_per_sm(c->rc) * c->num_sms;
-    const int granule = (flags & SFHE_EXEC_LAZY) ? c->rc.lazy_group : 1;
+    const UnitCosts costs = unit_costs(c, flags);
+    const int grid = costs.per_sm * costs.sms, granule = costs.group;
     const int longest = P.entries[0].count;
     if (grid <= 0 || P.out_entries >= 8 * (int64_t)grid || longest <= granule) return;
-    auto parts_of = [](int count, int u) { return count <= u ? 1 : (count + u - 1) / u; };
-    std::vector<double> cost;
-    double best = 0;
-    int best_u = 0, last_u = 0;
     double work = 0;
-    for (const Entry& e : P.entries) work += e.count + kRelinCost;
+    for (const Entry& e : P.entries)
+        if (e.count) work += costs.work(e.count) + costs.relin;
+    work *= costs.slowdown(costs.per_sm) / grid;
+    double best = 1e300;
+    int last_u = 0, best_u = 0;
     // candidates in steps of about 4/3: this runs on the host in one-shot calls
     for (int pieces = 1; pieces <= (longest + granule - 1) / granule && pieces <= 256; pieces += 1 + pieces / 3) {
         const int u = (((longest + granule - 1) / granule + pieces - 1) / pieces) * granule;
         if (u == last_u) continue;
         last_u = u;
         int64_t slots = 0;
-        cost.clear();
-        for (const Entry& e : P.entries) {
-            const int parts = parts_of(e.count, u);
-            if (parts > 1) slots += parts;
-            for (int p = 0; p < parts; p++)
-                cost.push_back(std::min(u, e.count - p * u) + (p == parts - 1 ? kRelinCost : 0.0) +
-                               (parts > 1 ? kPartCost : 0.0) + (p == parts - 1 && parts > 1 ? kPartCost * parts : 0.0));
-        }
+        for (const Entry& e : P.entries) slots += e.count > u ? (e.count + u - 1) / u : 0;
         if (slots > 2 * (int64_t)grid) break;
-        std::sort(cost.begin(), cost.end(), std::greater<double>());
-        const double t = schedule_length(cost, grid);
-        if (pieces == 1 || t < 0.97 * best) best = t, best_u = u;
-        if (best < 1.05 * work / grid) break;  // the chip is filled evenly
+        const double t = launch_length(P.entries, u, costs, best);
+        if (t < best) best = t, best_u = u;
+        if (best < 1.05 * work) break;  // the chip is filled evenly
     }
     if (best_u >= longest) return;
-    std::vector<Entry> units;
-    for (const Entry& e : P.entries) {
-        const int parts = parts_of(e.count, best_u), first_slot = P.slots;
-        for (int p = 0; p < parts; p++) {
-            Entry x = e;
-            x.first = e.first + p * best_u;
-            x.count = std::min(best_u, e.count - p * best_u);
-            x.parts = parts;
-            x.first_slot = parts > 1 ? first_slot : 0;
-            x.slot = parts > 1 ? first_slot + p : 0;
-            units.push_back(x);
-        }
-        if (parts > 1) P.slots += parts;
-    }
-    std::stable_sort(units.begin(), units.end(), [](const Entry& a, const Entry& b) { return a.count > b.count; });
+    std::vector<Entry> units = units_of(P.entries, best_u);
+    for (const Entry& x : units) P.slots += x.parts > 1;
     std::vector<int> last(P.slots, 0);  // by first slot
     for (size_t i = 0; i < units.size(); i++) {
         if (units[i].parts > 1) last[units[i].first_slot] = (int)i;
