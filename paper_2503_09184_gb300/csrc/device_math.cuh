@@ -365,13 +365,6 @@ SFHE_DEV int sample_gauss(u64 key, u64 slot, const u64* cdt)
 }
 // residue mod q of an integer between -q and q
 SFHE_DEV u64 small_residue(int v, u64 q) { return v < 0 ? q - (u64)(-v) : (u64)v; }
-// signed integer to its residue mod q
-SFHE_DEV u64 to_residue(long long v, u64 q)
-{
-    if (v >= 0) return (u64)v % q;
-    u64 r = (u64)(-v) % q;
-    return r ? q - r : 0;
-}
 
 // ------------------------------------------------- TMA bulk copies ---------
 // One-dimensional bulk copies global -> shared through the tensor memory

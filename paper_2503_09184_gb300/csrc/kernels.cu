@@ -236,7 +236,7 @@ cudaError_t launch_relin_accum(const RnsConsts& rc, const u64* U, const u64* rlk
 size_t persistent_scratch_words(const RnsConsts& rc)
 {
     const size_t N = rc.N, L = rc.L, K = rc.K;
-    const size_t w = 3 * L * N + 2 * N + (3 * K * N + 1) / 2;
+    const size_t w = 3 * L * N + (3 * K * N + 1) / 2;
     return (w + 31) & ~(size_t)31;  // 256-byte aligned slots
 }
 

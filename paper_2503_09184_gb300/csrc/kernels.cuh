@@ -719,7 +719,7 @@ struct PersistentTile {
 // limb for limb, to relinearising every product and adding.
 // Scratch per CTA: acc [3][L][N] uint64 (plain 64-bit sums: of the digits
 // D_j, canonical, exact for up to 1024 products; of d0 and d1 in [0, 3 q_i),
-// folded to canonical every 256 products), cacc [2][N] uint64, T [3][K][N]
+// folded to canonical every 256 products), T [3][K][N]
 // uint32 (x~_k, the inverse NTT's output).  queue[0] is the entry counter, queue[1] the error word (1: a
 // bulk copy did not complete within the wait bound).  mbarriers 0 and 1
 // track the operand pairs of stage T.  `entries` lists units of work: whole
@@ -748,8 +748,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
     __shared__ u32 s_tmem;
     const int tid = threadIdx.x;
     u64* base = scratch + (size_t)blockIdx.x * scratch_stride;
-    u64* cacc = base + (size_t)3 * L * N;                   // [2][N] u64, behind the sums [3][L][N]
-    u32* T = reinterpret_cast<u32*>(cacc + (size_t)2 * N);  // [3][K][N] u32
+    u32* T = reinterpret_cast<u32*>(base + (size_t)3 * L * N);  // [3][K][N] u32, behind the sums [3][L][N] u64
     const size_t ext_words = (size_t)2 * K * N;
     const size_t ct_words = (size_t)2 * L * N;
     const ulonglong2* key = reinterpret_cast<const ulonglong2*>(rlk);  // pairs, lane-interleaved
@@ -1429,6 +1428,7 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
             // within the registers the CTA is launched with; U and the sums
             // stay lane-interleaved until the output
             static_assert(NQ::SMEM_WORDS * 8 <= PP::SMEM, "shared memory of the looped transform");
+            static_assert((L + 2) * sizeof(u64) <= 3 * K * sizeof(u32), "a limb's transforms fit where x~ lay");
             u64* U = reinterpret_cast<u64*>(T);  // [L + 2][N], lane-interleaved
             for (int i = 0; i < L; i++) {
                 const Mod m = c.m[i];

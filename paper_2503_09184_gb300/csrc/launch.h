@@ -91,8 +91,6 @@ size_t rotate_batch_words(const RnsConsts& rc, long long n);
 cudaError_t launch_rotate_batch(const RnsConsts& rc, const u64* in, size_t in_stride, long long n, u32 g,
                                 const u64* key, const u64* key_sh, u64* out, size_t out_stride, u64* work,
                                 long long batch, cudaStream_t s);
-cudaError_t launch_rotate(const RnsConsts& rc, const u64* in, u32 g, const u64* key, const u64* key_sh, u64* out,
-                          u64* work, cudaStream_t s);
 // a bounded wait that runs out: sets queue[1] = 1 (selftest.cu)
 cudaError_t launch_wait_selftest(unsigned* queue, u32 tries, u64 limit_ns, cudaStream_t s);
 // multiplies per second of shoup32_lazy over all SMs (8 independent chains

@@ -432,16 +432,7 @@ cudaError_t launch_rotate_batch(const RnsConsts& rc, const u64* in, size_t in_st
     return cudaSuccess;
 }
 
-// Rotation of one ciphertext: a batch of one.  Work per ciphertext: P
-// [2][L][N], the digits [L][N] and their transforms [L][L][N] (uint64; the
-// callers' workspaces keep room for four more rows of L N words).
-size_t rotate_work_words(const RnsConsts& rc) { return (size_t)(2 + 3 + rc.L + 2) * rc.L * rc.N; }
-
-cudaError_t launch_rotate(const RnsConsts& rc, const u64* in, u32 g, const u64* key, const u64* key_sh, u64* out,
-                          u64* work, cudaStream_t s)
-{
-    const size_t ctw = (size_t)2 * rc.L * rc.N;
-    return launch_rotate_batch(rc, in, ctw, 1, g, key, key_sh, out, ctw, work, 1, s);
-}
+// per ciphertext: P [2][L][N], the digits [L][N] and their transforms [L][L][N] (uint64)
+size_t rotate_work_words(const RnsConsts& rc) { return (size_t)(2 + 1 + rc.L) * rc.L * rc.N; }
 
 }  // namespace sfhe
