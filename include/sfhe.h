@@ -519,13 +519,21 @@ void sfhe_host_plan_destroy(sfhe_host_plan* hp);
 /* The same products over caller-owned device memory (sfhe_matrix_view):
  * the caller allocates C's ciphertexts and the workspace, and picks the
  * execution mode.  Workspace (device bytes) for n matmuls A[m] x B[m] under
- * `flags`: */
+ * `flags`.  A PERSISTENT plan of few output entries (fewer than 8 per CTA)
+ * may share the products of an entry out over several units of work, which
+ * keeps all SMs busy; every such unit has a slot of 3 L N words for its sums,
+ * at most two slots per CTA (239 MB at N = 8192, L = 4 and 956 MB at
+ * N = 16384, L = 8 on 152 SMs), and they are part of this size.  A workspace
+ * that is too small for the slots but holds the rest is accepted: the plan
+ * then keeps whole entries, with the same results, later (up to 10 times for
+ * a single long entry). */
 sfhe_status sfhe_matmul_workspace_size(const sfhe_ctx* ctx, int32_t n, const sfhe_matrix_view* A,
                                        const sfhe_matrix_view* B, uint32_t flags, size_t* bytes);
 /* An upper bound of sfhe_matmul_workspace_size for any n <= max_matmuls
  * matmuls with at most max_entries output entries and max_products
  * products in all (a workspace a serving loop allocates once and reuses for
- * every batch).  Host only.  Errors: EINVAL, ESHAPE (negative bounds). */
+ * every batch); for PERSISTENT flags it holds the slots of shared-out entries
+ * at their maximum, or one per product if that is less.  Host only.  Errors: EINVAL, ESHAPE (negative bounds). */
 sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* ctx, int32_t max_matmuls, int64_t max_entries,
                                         int64_t max_products, uint32_t flags, size_t* bytes);
 /* C = A x B with the k-loop over every k: the naive dense loop of Alg. 1
@@ -556,8 +564,8 @@ sfhe_status sfhe_plan_create(sfhe_ctx* ctx, int32_t n, const sfhe_matrix_view* A
 sfhe_status sfhe_plan_execute(sfhe_plan* plan, void* stream);
 /* Synchronises `stream` and reads the status word of a matmul workspace
  * after a PERSISTENT execution: SFHE_ETIMEOUT if one of the kernel's bounded
- * waits for an operand copy ran out (the kernel then stopped early and C is
- * incomplete). */
+ * waits (for an operand copy, or at L = 8 for a matrix product of the
+ * rounding) ran out: the kernel then stopped early and C is incomplete. */
 sfhe_status sfhe_matmul_check(void* work, void* stream);
 /* Preemption of a persistent plan: the serving loop's continuous admission
  * (a request that arrives while a plan runs need not wait for the whole
@@ -566,17 +574,22 @@ sfhe_status sfhe_matmul_check(void* work, void* stream);
  * sfhe_plan_set_stop: `word` is the device address of one uint32 (NULL
  * clears it), which the caller owns and writes, e.g. with a copy on another
  * stream while the launch runs.  Every CTA of the plan's persistent launches
- * reads it before it takes its next output entry and takes none once it is
- * nonzero; no CTA waits on it, so a launch ends within one entry's time of
- * the word being set, the entries it took complete, C of the others is
- * untouched.  Errors: EINVAL (null plan, a PLAIN or GRAPH plan, misaligned).
+ * reads it before it takes its next unit of work (a whole output entry, or
+ * part of one where the plan shares its entries out; see
+ * sfhe_matmul_workspace_size) and takes none once it is nonzero; no CTA waits
+ * on it, so a launch ends within one unit's time of the word being set, with
+ * the units it took complete.  C of an entry is written when the entry's last
+ * unit is done: entries without a unit left are complete, C of the others is
+ * untouched, also where some of their units are done.  Errors: EINVAL (null
+ * plan, a PLAIN or GRAPH plan, misaligned).
  * sfhe_plan_progress: synchronises `stream` and reports how many output
- * entries, in the plan's execution order, the launches so far completed
- * (all of them after an execution that was not stopped).
- * sfhe_plan_resume: launches the plan again from its first entry not taken
- * (clear the word first); a stopped execution plus its resumptions write
+ * entries the launches so far completed (all of them after an execution that
+ * was not stopped); which ones is not reported.
+ * sfhe_plan_resume: launches the plan again from its first unit not taken
+ * (clear the word first); the sums of half-done entries stay in the
+ * workspace in between.  A stopped execution plus its resumptions write
  * the same C, limb for limb, as one execution.  sfhe_plan_execute restarts
- * from the first entry.  Errors: EINVAL (null plan, a PLAIN plan, resume
+ * from the first unit.  Errors: EINVAL (null plan, a PLAIN plan, resume
  * before the first execution), ECUDA. */
 sfhe_status sfhe_plan_set_stop(sfhe_plan* plan, const uint32_t* word);
 sfhe_status sfhe_plan_progress(const sfhe_plan* plan, int64_t* done, void* stream);
@@ -642,8 +655,8 @@ sfhe_status sfhe_ct_mul_relin(sfhe_ctx* ctx, const uint32_t* a_ext, const uint32
  * Rings whose scratch, 3 K N uint32 words (rounded up to 256 bytes) +
  * (3 L + (L+2) L) N uint64 words, exceeds the array are rejected with
  * SFHE_ENOMEM (N = 8192, L = 4 needs 3.8 MB and fits; N = 16384, L = 8
- * needs 19.5 MB and does not).  Nothing in the scratch has to start at
- * zero; `out` is cleared by the call.  All calls on one device share the
+ * needs 19.5 MB and does not).  Nothing in the scratch or in `out` has to
+ * start at zero.  All calls on one device share the
  * array: calls that overlap in time (other streams, other threads) race
  * and must be serialised by the caller. */
 sfhe_status sfhe_ct_mul_relin_static(sfhe_ctx* ctx, const uint32_t* a_ext, const uint32_t* b_ext, uint64_t* out,

@@ -1297,7 +1297,9 @@ extern "C" sfhe_status sfhe_matmul_check(void* work, void* stream)
     CUDA_TRY(cudaStreamSynchronize(as_stream(stream)));
     unsigned err = 0;
     CUDA_TRY(cudaMemcpy(&err, (char*)work + sizeof(unsigned), sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (err) return fail(SFHE_ETIMEOUT, "an operand copy of the persistent kernel did not complete within its wait bound");
+    if (err)
+        return fail(SFHE_ETIMEOUT, "an operand copy or a matrix product of the persistent kernel did not complete within "
+                                   "its wait bound");
     return SFHE_OK;
 }
 

@@ -72,18 +72,18 @@ SFHE_DEV u64 barrett_lazy(u64 hi, u64 lo, Mod m)
 typedef long long i64;
 SFHE_DEV int pm_c(u64 q) { return (int)(0u - (u32)q); }
 
-// a w mod q for |a| <= 2^62 and a prepared constant (w, w2): with
+// a w mod q for |a| <= 2^62.1 and a prepared constant (w, w2): with
 // a = a1 2^32 + a0 (a0 signed), a w = a0 w + a1 (2^32 w), and with the
 // constants split at bit 22 the sum is p0 + 2^22 p1 = p0 + 2^22 lo(p1) +
 // 2^54 hi(p1), whose last term folds to c hi(p1): five signed 32x32->64-bit
 // multiply-adds, no carries (Shoup's form of the same product takes ten
-// 32-bit multiplies and their carries).  |p1| < 2^62 + 2^61,
-// |p0| < 2^53 + 2^52; the result lies in (-2^54.6, 2^55.3) for any such a,
-// and within 2^55 for |a| <= 2^60.  A 32x32->64-bit multiply-add occupies
-// the issue of a scheduler for 4.25 cycles (measured, full chip), a 32-bit
-// one or a shift for 2.1, an add for 1.06: the product costs 26 cycles per
-// warp, Shoup's 34.  (Written with inline PTX: from C++ the signed products
-// were compiled to 47 cycles.)
+// 32-bit multiplies and their carries).  |p1| < 2^62 + 2^61.1,
+// |p0| < 2^53 + 2^52.1; the result lies in (-2^54.7, 2^55.4) for any such a,
+// and within 2^55 for |a| <= 2^60 and c < 2^22.4 (2^55.1 for any c < 2^23).
+// A 32x32->64-bit multiply-add occupies the issue of a scheduler for 4.25
+// cycles (measured, full chip), a 32-bit one or a shift for 2.1, an add for
+// 1.06: the product costs 26 cycles per warp, Shoup's 34.  (Written with
+// inline PTX: from C++ the signed products were compiled to 47 cycles.)
 SFHE_DEV i64 mad_wide(int a, int b, i64 c)
 {
     i64 d;
@@ -123,7 +123,7 @@ SFHE_DEV u64 pm_canon(i64 v, u64 q)
 }
 // The same arithmetic for a prime of any n bits, 32 < n <= 54, q = 2^n - c,
 // c < 2^23 (constants split at bit n - 32): |p1| and |p0| keep their bounds, so
-// the products stay within 2^55 as above however small q is.
+// the products stay within 2^55.1 (2^55.4) as above however small q is.
 SFHE_DEV int pm_bits(u64 q) { return 64 - __clzll((long long)q); }
 SFHE_DEV int pm_c_any(u64 q) { return (int)((1ULL << pm_bits(q)) - q); }
 SFHE_DEV i64 pm_mul_any(i64 a, u64 w, u64 w2, int c, int n)
@@ -133,7 +133,7 @@ SFHE_DEV i64 pm_mul_any(i64 a, u64 w, u64 w2, int c, int n)
     const i64 p0 = mad_wide(a1, (int)w2, mul_wide(a0, (int)w));
     return mad_wide((int)(p1 >> 32), c, p0) + (i64)((u64)(u32)p1 << (n - 32));
 }
-// one fold of |v| < 2^62: below 2^54 in magnitude (h c < 2^29 2^23)
+// one fold of |v| < 2^63: below 2^54.1 in magnitude (h c < 2^30 2^23 at n = 33, 2^9 2^23 at n = 54)
 SFHE_DEV i64 pm_fold_any(i64 v, int c, int n)
 {
     return mad_wide((int)(v >> n), c, (i64)((u64)v & ((1ULL << n) - 1)));

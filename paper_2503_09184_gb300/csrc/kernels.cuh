@@ -195,26 +195,7 @@ SFHE_DEV void scale_round_out(const u32 (&xt)[M][K], const u32 (&v)[M], const u6
     }
 }
 
-// Exact round(t x / Q) mod q_i for M tensor coefficients x, each given by
-// x~_k = [x_k (B/b_k)^-1]_{b_k} at xt32[m][k * stride] (canonical, k < K; the
-// tensor stage's inverse NTT produces them):
-//   x = sum_k x~_k (B/b_k) - v B,
-//   v = round(sum_k x~_k / b_k)  (sum_k x~_k / b_k = v + x / B, |x| / B < 1/4);
-//   with t (B/b_k) = alpha_k Q + r_k and t B = alpha_B Q + r_B,
-//   t x / Q = sum_k x~_k alpha_k - v alpha_B + F,  F = (sum_k x~_k r_k - v r_B) / Q,
-// so round(t x / Q) = sum_k x~_k alpha_k - v alpha_B + round(F).  F + K > 0
-// is estimated as G / 2^64 with G = sum_k x~_k rho_k - v rho_B + K 2^64,
-// rho = floor(r 2^64 / Q); with the exact rho_k the true value lies in
-// (G - K, G + K 2^30) / 2^64,
-// so round(F) + K = floor((G + 2^63) / 2^64) unless that interval crosses
-// the rounding point, where the decision is taken exactly (Q is odd: no ties).
-// Every product is one 32x32-bit multiply into a 64-bit sum without carries:
-// G takes rho_k without its low 6 bits, in two 29-bit parts (products below
-// 2^59), which widens the band to (G - K, G + K 2^37); the 54-bit
-// [alpha_k]_{q_i} is split at bit 27 (below 2^62).  The M coefficients are
-// independent; they are interleaved for instruction-level parallelism.
-// LAZY: d[m][i] in [0, 3 q_i) (congruent, one Barrett step without the final
-// subtractions) instead of canonical.
+// both halves
 template <int L, int K, int M, bool LAZY = false>
 SFHE_DEV void scale_round_m(const u32* const (&x32)[M], size_t stride, const RnsConsts& c, u64 (&d)[M][L])
 {
@@ -718,10 +699,12 @@ struct PersistentTile {
 // so the relinearisation NTTs run once per entry; the result is identical,
 // limb for limb, to relinearising every product and adding.
 // Scratch per CTA: acc [3][L][N] uint64 (plain 64-bit sums: of the digits
-// D_j, canonical, exact for up to 1024 products; of d0 and d1 in [0, 3 q_i),
-// folded to canonical every 256 products), T [3][K][N]
-// uint32 (x~_k, the inverse NTT's output).  queue[0] is the entry counter, queue[1] the error word (1: a
-// bulk copy did not complete within the wait bound).  mbarriers 0 and 1
+// D_j, canonical, exact for up to 1024 products; of d0 and d1, congruent: in
+// [0, 3 q_i) and reduced to canonical every 256 products, or, rounded on the
+// tensor cores, below 2^55.3 and folded below 2^54.1 every 255), T [3][K][N]
+// uint32 (x~_k, the inverse NTT's output).  queue[0] is the unit counter,
+// queue[1] the error word (1: a bulk copy or a matrix product did not complete
+// within the wait bound).  mbarriers 0 and 1
 // track the operand pairs of stage T.  `entries` lists units of work: whole
 // output entries, or (few entries, see split_entries in api.cu) parts of an
 // entry's products whose sums meet in `partial` / `finished`.
@@ -1376,12 +1359,14 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
             __syncthreads();
         }
         // stage R.  The forward NTT leaves slot tid * R + v of every polynomial
-        // with thread tid, so the key products and the output are private to
-        // a thread, and the key and C are accessed with 16-byte vectors.  Up
-        // to N = 8192 the sums [2][N] live in the idle operand slots (element
-        // v of thread tid at v * NTH + tid, free of bank conflicts).  At
-        // N = 16384 they do not fit: the L + 2 transforms of a limb go to the
-        // idle tensor scratch and one pass forms both sums in registers.
+        // with thread tid, and the key is stored so that a warp reads its pairs
+        // at consecutive addresses (lane-interleaved, 16-byte loads): the key
+        // products and the sums are private to a thread.  Up to N = 8192 the
+        // sums [2][N] live in the idle operand slots (element v of thread tid
+        // at v * NTH + tid, free of bank conflicts); at N = 16384 they do not
+        // fit: the L + 2 transforms of a limb go to the idle tensor scratch and
+        // one pass forms both sums in registers.  C is written coalesced,
+        // through one more exchange.
         if constexpr (PP::STAGED) {
             u64* cs = reinterpret_cast<u64*>(smb + PP::EXB);
             for (int i = 0; i < L; i++) {

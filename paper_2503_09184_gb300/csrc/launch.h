@@ -46,7 +46,7 @@ struct PersistentArgs {
     const Entry* entries;
     int n_entries;
     const int2* rowlist;
-    const u64* rlk;  // in pm_mul's form: all w's, then all w2's
+    const u64* rlk;  // in pm_mul's form: pairs (w, w2)
     u64* scratch;
     size_t scratch_stride;
     unsigned* queue;

@@ -64,9 +64,10 @@ struct Arith64 {
 template <bool ANY>  // ANY: a prime of any 33 to 54 bits, else 54 bits
 struct ArithPm {
     using W = u64;
-    // inverse: inputs are below 2^54; after s stages without a fold the sums
-    // are below 2^(54+s), the differences fed to the product below
-    // 2^(54+s): eight stages stay within its range
+    // inverse: with inputs in [0, 2^55), words not yet multiplied are below
+    // 2^(55+s) after s stages and products, within 2^55.1 at first, stay below
+    // 2^(54.1+s), so that the difference fed to stage s's product is within
+    // 2^(54.1+s): eight stages stay within 64-bit words (and the folds' range)
     static constexpr int FOLD_STAGES = 8;
     static constexpr bool PAIRS = true;  // twiddle layout: see tw_pair
     SFHE_DEV static W mul(W a, W w, W w2, W q)
@@ -579,8 +580,11 @@ struct NttT {
         }
     }
 
-    // x: run_idx layout in ([0, 2q)), inv_out_idx layout out ([0, 2q)).
-    // (ni, nis) = N^-1 and its Shoup companion; (wl, wls) = ipsi_rev[1] N^-1.
+    // x: run_idx layout in, inv_out_idx layout out.  Arith64 and Arith32 take
+    // and leave [0, 2q); ArithPm takes [0, 2^55) (eight stages without a fold:
+    // sums below 2^63, differences fed to a product below 2^62.1) and leaves
+    // signed products, within 2^55.4, for pm_canon.
+    // (ni, nis) = N^-1 prepared for the policy's product; (wl, wls) = ipsi_rev[1] N^-1.
     // sm holds NP * SMEM_WORDS words.
     template <int NP>
     SFHE_DEV static void inverse_m(W (&x)[NP][R], W* sm, int tid, const W* tw, W q, W ni, W nis, W wl, W wls)

@@ -19,15 +19,19 @@
 // Why and where: the CUDA-core form spends 2 K (L + 1) wide multiplies (4.25
 // issue cycles each) per coefficient, 540 at L = 8 (K = 30), where this one
 // spends about 10 (L + 1): as a contraction of length 4 K with 6 L + 7 columns
-// its products cost the tensor pipe a few per cent of the stage.  At L = 8,
-// N = 16384 the stage was a third of the kernel: two 32 x 64 x 16 matmuls at
-// 60% zeros 267 -> 241 ms (GB300; 0.92 -> 0.83 of one earlier build timed
-// beside both).  At L <= 4 (K <= 16) the two forms issue about as many
-// instructions, 450 per coefficient and warp, and the stage waits for its
-// residues and sums instead (2.3 MB of scratch per CTA, more than the CTAs'
-// share of L2): measured with byte subnormals, bulk-copied residues and
-// double-buffered tiles 64^3 gained 2.5% and the small ring (N = 4096) lost
-// 20%, so those rings keep the CUDA-core form.
+// its products cost the tensor pipe a few per cent of the stage, a third of
+// the kernel at L = 8.  Plans of 50% zeros before the 64-bit folds and this
+// rounding against now (GB300): N = 16384, 32 x 64 x 16, 199.4 -> 168.9 ms;
+// N = 8192, 32 x 32 x 16, 51.0 -> 40.1 ms; N = 4096, 32 x 32 x 32, 45.8 ->
+// 39.9 ms, there with one CTA on an SM in place of two (the runtime reports
+// one for any kernel that allocates tensor memory).  Two 32 x 64 x 16 matmuls
+// at 60% zeros: 294 -> 246 ms, of which this rounding 267 -> 241 when it came.
+// At L <= 4 (K <= 16) the two forms issue about as many instructions, 450 per
+// coefficient and warp, and the stage waits for its residues and sums instead
+// (2.3 MB of scratch per CTA, more than the CTAs' share of L2): measured with
+// byte subnormals, bulk-copied residues and double-buffered tiles 64^3 gained
+// 2.5% and the small ring (N = 4096) lost 20%, so those rings keep the
+// CUDA-core form.
 //
 // The left operand is written to tensor memory by the thread that owns the
 // row (no shared-memory layout), the right one sits in shared memory
