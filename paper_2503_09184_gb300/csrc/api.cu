@@ -743,7 +743,7 @@ UnitCosts unit_costs(const sfhe_ctx* c, uint32_t flags)
     UnitCosts k;
     k.group = (flags & SFHE_EXEC_LAZY) ? c->rc.lazy_group : 1;
     k.sms = c->num_sms;
-    k.per_sm = persistent_ctas_per_sm(c->rc);
+    k.per_sm = persistent_ctas_per_sm(c->rc, (flags & SFHE_EXEC_LAZY) != 0);
     k.threads = c->rc.N / ext_interleave(c->rc.logN);
     k.relin = 0.3 + 1.45 * c->rc.L * (c->rc.L + 2) / (3.0 * c->rc.K);
     return k;
@@ -947,7 +947,7 @@ Layout layout_of(const sfhe_ctx* c, const sfhe_plan& P, uint32_t flags, int* gri
     *grid_out = 0;
     *stride_out = 0;
     if (flags & SFHE_EXEC_PERSISTENT) {
-        const int per_sm = persistent_ctas_per_sm(c->rc);
+        const int per_sm = persistent_ctas_per_sm(c->rc, (flags & SFHE_EXEC_LAZY) != 0);
         int grid = per_sm * c->num_sms;
         grid = (int)std::min<size_t>((size_t)grid, std::max<size_t>(1, P.entries.size()));
         const size_t stride = persistent_scratch_words(c->rc);
@@ -1382,7 +1382,7 @@ extern "C" sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* c, int32_t ma
     off += align256((size_t)max_products * sizeof(int2));
     const size_t N = c->rc.N, L = c->rc.L, K = c->rc.K;
     if (flags & SFHE_EXEC_PERSISTENT) {
-        const size_t grid = (size_t)persistent_ctas_per_sm(c->rc) * c->num_sms;
+        const size_t grid = (size_t)persistent_ctas_per_sm(c->rc, (flags & SFHE_EXEC_LAZY) != 0) * c->num_sms;
         off += align256(grid * persistent_scratch_words(c->rc) * 8);
         // split_entries: at most 2 units per CTA share entries out, of at
         // least one product each; more units than entries in the list
@@ -1741,7 +1741,7 @@ static const long long kTermRotBatch = 128;
 // term_batch(c): three rounds of the persistent kernel's grid.
 static int64_t term_batch(const sfhe_ctx* c)
 {
-    return 3 * (int64_t)std::max(1, persistent_ctas_per_sm(c->rc) * c->num_sms);
+    return 3 * (int64_t)std::max(1, persistent_ctas_per_sm(c->rc, false) * c->num_sms);
 }
 
 // workspace of sfhe_matmul_chunked: the batched rotation scratch; five

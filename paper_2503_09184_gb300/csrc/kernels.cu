@@ -240,12 +240,12 @@ size_t persistent_scratch_words(const RnsConsts& rc)
     return (w + 31) & ~(size_t)31;  // 256-byte aligned slots
 }
 
-int persistent_ctas_per_sm(const RnsConsts& rc)
+int persistent_ctas_per_sm(const RnsConsts& rc, bool grouped)
 {
     switch (rc.logN) {
-    case 12: return persistent_occupancy<12>(rc.L);
-    case 13: return persistent_occupancy<13>(rc.L);
-    case 14: return persistent_occupancy<14>(rc.L);
+    case 12: return persistent_occupancy<12>(rc.L, grouped);
+    case 13: return persistent_occupancy<13>(rc.L, grouped);
+    case 14: return persistent_occupancy<14>(rc.L, grouped);
     default: return 0;
     }
 }

@@ -61,7 +61,7 @@ struct PersistentArgs {
     float l2_hit_ratio;
 };
 template <int LOGN>
-int persistent_occupancy(int L);
+int persistent_occupancy(int L, bool grouped);
 template <int LOGN>
 cudaError_t persistent_launch(const RnsConsts& rc, const PersistentArgs& a, cudaStream_t s);
 // the tuned stage-S variants 1 and 2 of the rings that have them
@@ -70,7 +70,7 @@ template <int LOGN, int L, int V>
 cudaError_t persistent_launch_variant(const RnsConsts& rc, const PersistentArgs& a, cudaStream_t s);
 // words of the per-CTA scratch of the persistent kernel (uint64 units)
 size_t persistent_scratch_words(const RnsConsts& rc);
-int persistent_ctas_per_sm(const RnsConsts& rc);
+int persistent_ctas_per_sm(const RnsConsts& rc, bool grouped);
 // tile variants of the per-product persistent kernel at this ring (1: the
 // default only; 3 where the tuner has candidates) and a name for each
 int persistent_variants(const RnsConsts& rc);

@@ -2,6 +2,6 @@
 #include "persistent_impl.cuh"
 
 namespace sfhe {
-template int persistent_occupancy<13>(int);
+template int persistent_occupancy<13>(int, bool);
 template cudaError_t persistent_launch<13>(const RnsConsts&, const PersistentArgs&, cudaStream_t);
 }  // namespace sfhe

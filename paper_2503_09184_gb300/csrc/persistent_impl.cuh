@@ -17,26 +17,27 @@ constexpr bool has_variants(int logN, int L)
 // rings with the NTT-form variants 3 and 4 (persistent_tuned_13b.cu)
 constexpr bool has_ntt_variants(int logN, int L) { return logN == 13 && L == 4; }
 
-template <int LOGN, int L>
+// of the mode's own instance: at N = 4096 with L = 3 and 4 the grouped one
+// takes 182 to 188 registers, and one CTA of it fits where two of the other do
+template <int LOGN, int L, bool GROUPED>
 static int occupancy_of()
 {
     int blocks = 0;
     const size_t smem = PersistentPlan<LOGN, L>::SMEM;
-    if (allow_smem(k_matmul_persistent<LOGN, L, false, 0>, smem) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_matmul_persistent<LOGN, L, false, 0>, NttGeom<LOGN>::T32::NT,
-                                                      smem) != cudaSuccess)
-        return 0;
+    auto* kern = k_matmul_persistent<LOGN, L, GROUPED, 0>;
+    if (allow_smem(kern, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, NttGeom<LOGN>::T32::NT, smem) != cudaSuccess) return 0;
     return blocks;
 }
 
 template <int LOGN>
-int persistent_occupancy(int L)
+int persistent_occupancy(int L, bool grouped)
 {
     switch (L) {
-    case 2: return occupancy_of<LOGN, 2>();
-    case 3: return occupancy_of<LOGN, 3>();
-    case 4: return occupancy_of<LOGN, 4>();
-    case 8: return occupancy_of<LOGN, 8>();
+    case 2: return grouped ? occupancy_of<LOGN, 2, true>() : occupancy_of<LOGN, 2, false>();
+    case 3: return grouped ? occupancy_of<LOGN, 3, true>() : occupancy_of<LOGN, 3, false>();
+    case 4: return grouped ? occupancy_of<LOGN, 4, true>() : occupancy_of<LOGN, 4, false>();
+    case 8: return grouped ? occupancy_of<LOGN, 8, true>() : occupancy_of<LOGN, 8, false>();
     default: return 0;
     }
 }

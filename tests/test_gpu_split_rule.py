@@ -39,3 +39,21 @@ def test_entries_are_shared_out_where_sms_would_idle(N, L):
     plan.execute()
     assert (coeff_of(api, ctx, plan.Cs[0]) == coeff_of(api, ctx, api.matmul(ctx, Ae, Be, mode="plain"))).all()
     plan.close()
+
+
+@pytest.mark.parametrize("L", [3, 4])
+def test_a_grouped_launch_has_as_many_ctas_as_are_resident(L):
+    """N = 4096, L = 3 and 4: two CTAs of the per-product kernel fit on an SM,
+    one of the grouped kernel (its registers); a launch of more would run the
+    rest after the others, and the schedule would count on them"""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for mode, per_sm in (("persistent", 2), ("lazy", 1)):
+        api, ctx, Ae, Be, plan = _plan(4096, L, 20, 3, 20, mode)
+        assert plan.stats["entries"] == 400 and plan.stats["ctas"] == per_sm * sms, mode
+        plan.execute()
+        if mode == "lazy":  # one group per entry
+            want = ((W.sparse_int_matrix(20, 3, 0.0, -16, 16, 91) @ W.dense_int_matrix(3, 20, -16, 16, 92) + 32768)
+                    % W.T_PLAIN) - 32768
+            assert (api.decrypt(ctx, plan.Cs[0]) == want).all()
+        plan.close()
