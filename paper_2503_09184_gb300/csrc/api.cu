@@ -885,20 +885,27 @@ void split_entries(const sfhe_ctx* c, sfhe_plan& P, uint32_t flags)
     const int grid = costs.per_sm * costs.sms, granule = costs.group;
     const int longest = P.entries[0].count;
     if (grid <= 0 || P.out_entries >= 8 * (int64_t)grid || longest <= granule) return;
+    // candidates in steps of about 4/3, as far as their slots are within the
+    // bound: this runs on the host in one-shot calls
+    std::vector<int> candidates;
+    for (int pieces = 1; pieces <= (longest + granule - 1) / granule && pieces <= 256; pieces += 1 + pieces / 3) {
+        const int u = (((longest + granule - 1) / granule + pieces - 1) / pieces) * granule;
+        if (!candidates.empty() && u == candidates.back()) continue;
+        int64_t slots = 0;
+        for (const Entry& e : P.entries) slots += e.count > u ? (e.count + u - 1) / u : 0;
+        if (slots > 2 * (int64_t)grid) break;
+        candidates.push_back(u);
+    }
+    // most plans of several entries per CTA end here (1060 entries of 7
+    // products on 304 CTAs, a one-shot call of 3.8 ms: 77 us less)
+    if (candidates.size() < 2) return;
     double work = 0;
     for (const Entry& e : P.entries)
         if (e.count) work += costs.work(e.count) + costs.relin;
     work *= costs.slowdown(costs.per_sm) / grid;
     double best = 1e300;
-    int last_u = 0, best_u = 0;
-    // candidates in steps of about 4/3: this runs on the host in one-shot calls
-    for (int pieces = 1; pieces <= (longest + granule - 1) / granule && pieces <= 256; pieces += 1 + pieces / 3) {
-        const int u = (((longest + granule - 1) / granule + pieces - 1) / pieces) * granule;
-        if (u == last_u) continue;
-        last_u = u;
-        int64_t slots = 0;
-        for (const Entry& e : P.entries) slots += e.count > u ? (e.count + u - 1) / u : 0;
-        if (slots > 2 * (int64_t)grid) break;
+    int best_u = longest;
+    for (int u : candidates) {
         const double t = launch_length(P.entries, u, costs, best);
         if (t < best) best = t, best_u = u;
         if (best < 1.05 * work) break;  // the chip is filled evenly
