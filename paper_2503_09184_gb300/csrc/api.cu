@@ -132,7 +132,7 @@ struct sfhe_plan {
     cudaGraphExec_t gexec;
     int variant;  // tile variant of the persistent kernel
     const unsigned* d_stop;  // preemption word of the persistent launches (nullable)
-    bool launched;           // an execution has set the entry counter
+    bool launched;           // an execution has set the unit counter
 };
 
 extern "C" const char* sfhe_last_error(void) { return g_last_error.c_str(); }
@@ -1057,7 +1057,8 @@ sfhe_status tune_variants(sfhe_plan* P, cudaStream_t s)
     // during an execution
     unsigned err = 0;
     CUDA_TRY(cudaMemcpy(&err, P->d_queue + 1, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (err) return fail(SFHE_ETIMEOUT, "an operand copy did not complete within its wait bound (tile tuning)");
+    if (err)
+        return fail(SFHE_ETIMEOUT, "an operand copy or a matrix product did not complete within its wait bound (tile tuning)");
     c->tuned_variant = best_v;
     return SFHE_OK;
 }
@@ -1282,7 +1283,7 @@ extern "C" sfhe_status sfhe_plan_resume(sfhe_plan* P, void* stream)
     if (!P) return fail(SFHE_EINVAL, "null plan");
     if (!(P->flags & SFHE_EXEC_PERSISTENT)) return fail(SFHE_EINVAL, "only PERSISTENT plans resume");
     if (!P->launched) return fail(SFHE_EINVAL, "resume before the plan's first execution");
-    // the entry counter is left as the stopped launch left it: the entries
+    // the unit counter is left as the stopped launch left it: the units
     // below it are complete, the rest are taken from it on
     if (P->entries.empty()) return SFHE_OK;
     CUDA_TRY(launch_persistent(P->ctx->rc, persistent_args(P, (int)P->entries.size(), P->variant), as_stream(stream)));

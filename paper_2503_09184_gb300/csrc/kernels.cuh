@@ -688,8 +688,8 @@ struct PersistentTile {
 #define SFHE_WAIT_TRIES (1u << 26)
 #define SFHE_WAIT_NS 1000000000ull
 
-// One CTA per output entry at a time, taken from a queue in descending
-// product count.  Per product (per rounding group of mm.group products in the
+// A CTA takes one unit of work at a time (an output entry, or part of one: see
+// below) from a queue in descending product count.  Per product (per rounding group of mm.group products in the
 // grouped accumulate-then-round mode): stage T (tensor + 3K inverse NTTs over B into
 // the CTA's scratch), stage S (exact scale-and-round to Q, then the sums of
 // d0, d1 and of the digits D_j over the entry's products).  Per entry,
@@ -803,9 +803,9 @@ __global__ void __launch_bounds__(NttGeom<LOGN>::T32::NT) k_matmul_persistent(
 
     for (;;) {
         __syncthreads();
-        // a set stop word ends the launch at this entry boundary: the CTA
-        // takes no entry (it is never waited on), so queue[0] stays the
-        // number of entries taken and a later launch resumes from there
+        // a set stop word ends the launch at this boundary of units: the CTA
+        // takes none (it is never waited on), so queue[0] stays the number of
+        // units taken and a later launch resumes from there
         if (tid == 0)
             s_entry = (stop && *reinterpret_cast<const volatile unsigned*>(stop)) ? n_entries
                                                                                    : (int)atomicAdd(queue, 1u);

@@ -16,9 +16,9 @@ round-robin shares are the alternatives), so requests that
 arrive while others are on the GPU join the next wave and their products
 overlap with those already running.  With preemption (GpuExecutor's
 preempt) a request that arrives while a wave runs stops that wave at its
-next output-entry boundary (the plan's stop word): the newcomer is admitted,
-a wave over its rows runs, and the stopped wave resumes from its first entry
-not taken.  Every output entry is computed by exactly one wave from its own
+next unit boundary (the plan's stop word; a unit is an output entry or part
+of one): the newcomer is admitted, a wave over its rows runs, and the stopped
+wave resumes from its first unit not taken.  Every output entry is computed by exactly one wave from its own
 products, so a request's result is the same limb for limb alone and in any
 mix, stopped or not.
 
@@ -357,7 +357,7 @@ class GpuExecutor:
 
     def finish_wave(self, w: Wave, within_s: float | None = None) -> bool:
         """wait for the wave; if within_s (seconds) passes first, stop it at
-        its next entry boundary.  True once every entry is done (the plan is
+        its next unit boundary.  True once every entry is done (the plan is
         released), False if it stopped short (resume_wave continues it)."""
         torch, S = self.torch, self.S
         deadline = None if within_s is None or not self.preempt else time.perf_counter() + within_s
