@@ -871,8 +871,8 @@ KERNEL_SOURCES = ("kernels.cuh", "ntt.cuh", "device_math.cuh", "rns.h", "launch.
                   "persistent_tuned_13.cu", "persistent_tuned_13b.cu", "persistent_tuned_14.cu", "round_mma.cuh",
                   "round_shape.h")
 TRAFFIC = {  # (source hash, workload) -> (bytes per launch, profile summary)
-    ("a6654f27039fa051", "sweep-64x64x64-s0.5"): (715.07e9, "profiles/matmul_persistent_sweep64x64x64_s0.5_dram.md"),
-    ("a6654f27039fa051", "sweep-64x64x64-s0.5-lazy"): (170.46e9,
+    ("7b2564796d2fd085", "sweep-64x64x64-s0.5"): (707.16e9, "profiles/matmul_persistent_sweep64x64x64_s0.5_dram.md"),
+    ("7b2564796d2fd085", "sweep-64x64x64-s0.5-lazy"): (148.42e9,
                                                        "profiles/matmul_persistent_grouped_sweep64x64x64_s0.5_dram.md"),
 }
 
