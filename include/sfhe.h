@@ -536,6 +536,10 @@ sfhe_status sfhe_matmul_workspace_size(const sfhe_ctx* ctx, int32_t n, const sfh
  * at their maximum, or one per product if that is less.  Host only.  Errors: EINVAL, ESHAPE (negative bounds). */
 sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* ctx, int32_t max_matmuls, int64_t max_entries,
                                         int64_t max_products, uint32_t flags, size_t* bytes);
+/* The same without the slots of shared-out entries: enough for every such
+ * batch with whole entries, for a caller that is short of device memory. */
+sfhe_status sfhe_matmul_workspace_bound_whole(const sfhe_ctx* ctx, int32_t max_matmuls, int64_t max_entries,
+                                              int64_t max_products, uint32_t flags, size_t* bytes);
 /* C = A x B with the k-loop over every k: the naive dense loop of Alg. 1
  * (Sec. 3.3.1), each product multiplied, relinearised and added (A must
  * store every element: DENSE or MASK; masks are ignored). */

@@ -1376,8 +1376,8 @@ static sfhe_status size_impl(const sfhe_ctx* c, int32_t n, const sfhe_matrix_vie
     return SFHE_OK;
 }
 
-extern "C" sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* c, int32_t max_matmuls, int64_t max_entries,
-                                                   int64_t max_products, uint32_t flags, size_t* bytes)
+static sfhe_status bound_impl(const sfhe_ctx* c, int32_t max_matmuls, int64_t max_entries, int64_t max_products,
+                              uint32_t flags, bool share, size_t* bytes)
 {
     if (!c || !bytes) return fail(SFHE_EINVAL, "null argument");
     if (max_matmuls < 0 || max_entries < 0 || max_products < 0) return fail(SFHE_ESHAPE, "negative bound");
@@ -1394,13 +1394,25 @@ extern "C" sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* c, int32_t ma
         off += align256(grid * persistent_scratch_words(c->rc) * 8);
         // split_entries: at most 2 units per CTA share entries out, of at
         // least one product each; more units than entries in the list
-        const size_t slots = std::min<size_t>(2 * grid, (size_t)max_products);
+        const size_t slots = share ? std::min<size_t>(2 * grid, (size_t)max_products) : 0;
         off += align256(slots * sizeof(unsigned)) + align256(slots * sizeof(Entry)) + slots * partial_words(c->rc) * 8;
     }
     if (flags & SFHE_EXEC_PLAIN)
         off += align256(3 * K * N * 4) + align256(3 * L * N * 8) + align256((L + 2) * L * N * 8);
     *bytes = off;
     return SFHE_OK;
+}
+
+extern "C" sfhe_status sfhe_matmul_workspace_bound(const sfhe_ctx* c, int32_t max_matmuls, int64_t max_entries,
+                                                   int64_t max_products, uint32_t flags, size_t* bytes)
+{
+    return bound_impl(c, max_matmuls, max_entries, max_products, flags, true, bytes);
+}
+
+extern "C" sfhe_status sfhe_matmul_workspace_bound_whole(const sfhe_ctx* c, int32_t max_matmuls, int64_t max_entries,
+                                                         int64_t max_products, uint32_t flags, size_t* bytes)
+{
+    return bound_impl(c, max_matmuls, max_entries, max_products, flags, false, bytes);
 }
 
 extern "C" sfhe_status sfhe_matmul_workspace_size(const sfhe_ctx* c, int32_t n, const sfhe_matrix_view* A,

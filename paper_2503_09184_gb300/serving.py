@@ -263,7 +263,9 @@ class GpuExecutor:
     allocated once and reused: one, or two with preempt (a stopped wave keeps
     its plan and workspace while the wave that stopped it runs).  Their bytes
     (reserved_bytes) come out of the HBM budget before any request is
-    admitted.  setup_s and kernel_s add up the waves' plan set-up (work-list
+    admitted; they include the slots of waves whose entries are shared out
+    (up to 239 MB a workspace at N = 8192, L = 4), which whole_entries() gives
+    up.  setup_s and kernel_s add up the waves' plan set-up (work-list
     build and upload) and their persistent launches."""
 
     def __init__(self, ctx, stream=None, lazy: bool = False, wave_products: int = 40000, max_blocks: int = 1024,
@@ -281,11 +283,13 @@ class GpuExecutor:
         self.a_cache = {}
         self.admit_s = {}
         self.max_blocks = max_blocks
+        self.wave_products = wave_products
         self.preempt = preempt
         n = S.sfhe_matmul_workspace_bound(ctx.h, max_blocks, wave_products, wave_products, self.flags)
         self.works = [torch.empty(n, dtype=torch.uint8, device="cuda") for _ in range(2 if preempt else 1)]
         self.free = list(range(len(self.works)))
         self.reserved_bytes = n * len(self.works)
+        self.whole = False
         if preempt:
             # the stop word (device) and its set value (pinned host), written
             # on a side stream while a wave runs
@@ -294,6 +298,20 @@ class GpuExecutor:
             self.side = torch.cuda.Stream()
         self.setup_s, self.kernel_s = 0.0, 0.0
         self.stops = 0
+
+    def whole_entries(self):
+        """give up the workspaces' slots of shared-out entries: waves then run
+        whole entries (the same results; waves of few entries take longer)."""
+        S, torch = self.S, self.torch
+        n = S.sfhe_matmul_workspace_bound_whole(self.ctx.h, self.max_blocks, self.wave_products, self.wave_products,
+                                                self.flags)
+        count = len(self.works)
+        assert len(self.free) == count, "a wave is running"
+        self.stream.synchronize()
+        self.works = []
+        self.works = [torch.empty(n, dtype=torch.uint8, device="cuda") for _ in range(count)]
+        self.reserved_bytes = n * count
+        self.whole = True
 
     def admit(self, req: Request):
         """encrypt and lift the request's operands on the device (the client's
@@ -341,7 +359,11 @@ class GpuExecutor:
         parts = [self._rows(req, r0, r1) for req, r0, r1 in blocks]
         As, Bs, Cs = [p[0] for p in parts], [p[1] for p in parts], [p[2] for p in parts]
         slot = self.free.pop(0)
-        need = S.sfhe_matmul_workspace_size(self.ctx.h, [a.desc() for a in As], [b.desc() for b in Bs], self.flags)
+        if self.whole:
+            need = S.sfhe_matmul_workspace_bound_whole(
+                self.ctx.h, len(parts), sum(c.nct for c in Cs), sum(a.nct * b.cols for a, b, _ in parts), self.flags)
+        else:
+            need = S.sfhe_matmul_workspace_size(self.ctx.h, [a.desc() for a in As], [b.desc() for b in Bs], self.flags)
         # a wave of unusually many empty rows may need more than the bound
         work = self.works[slot] if need <= self.works[slot].numel() else torch.empty(need, dtype=torch.uint8,
                                                                                      device="cuda")
@@ -424,7 +446,13 @@ def serve(requests: list[Request], executor, budget_bytes: int, wave_products: i
     one entry's time plus its own work.  Without them every wave runs to
     completion (run_wave)."""
     # the executor's standing device memory (its matmul workspaces) is not
-    # available to requests
+    # available to requests; no request is rejected for the sake of the slots
+    # that only make waves of few entries faster
+    def fits(reserved):
+        s = Scheduler(budget_bytes - reserved, wave_products, ct_bytes, ext_bytes, order)
+        return all(request_bytes(r, ct_bytes, ext_bytes) <= s.budget or s.column_tiles(r) for r in requests)
+    if hasattr(executor, "whole_entries") and not fits(executor.reserved_bytes):
+        executor.whole_entries()
     sched = Scheduler(budget_bytes - getattr(executor, "reserved_bytes", 0), wave_products, ct_bytes, ext_bytes,
                       order)
     pending = deque(sorted(requests, key=lambda r: r.arrival))

@@ -79,6 +79,7 @@ _SIGS = {
     "sfhe_export_relin_key": ([_vp, _vp, _vp], ctypes.c_int),
     "sfhe_matmul_workspace_size": ([_vp, _i32, _P(sfhe_matrix_view), _P(sfhe_matrix_view), _u32, _P(_sz)], ctypes.c_int),
     "sfhe_matmul_workspace_bound": ([_vp, _i32, _i64, _i64, _u32, _P(_sz)], ctypes.c_int),
+    "sfhe_matmul_workspace_bound_whole": ([_vp, _i32, _i64, _i64, _u32, _P(_sz)], ctypes.c_int),
     "sfhe_matmul_dense_view": ([_vp, _P(sfhe_matrix_view), _P(sfhe_matrix_view), _P(sfhe_matrix_view), _u32, _vp, _sz, _vp], ctypes.c_int),
     "sfhe_matmul_sparse_view": ([_vp, _P(sfhe_matrix_view), _P(sfhe_matrix_view), _i32, _P(sfhe_matrix_view), _u32, _vp, _sz, _vp],
                            ctypes.c_int),
@@ -338,6 +339,13 @@ def sfhe_matmul_workspace_size(ctx: int, A: list, B: list, flags: int) -> int:
 def sfhe_matmul_workspace_bound(ctx: int, max_matmuls: int, max_entries: int, max_products: int, flags: int) -> int:
     b = ctypes.c_size_t()
     _check(lib().sfhe_matmul_workspace_bound(ctx, max_matmuls, max_entries, max_products, flags, ctypes.byref(b)))
+    return b.value
+
+
+def sfhe_matmul_workspace_bound_whole(ctx: int, max_matmuls: int, max_entries: int, max_products: int,
+                                      flags: int) -> int:
+    b = ctypes.c_size_t()
+    _check(lib().sfhe_matmul_workspace_bound_whole(ctx, max_matmuls, max_entries, max_products, flags, ctypes.byref(b)))
     return b.value
 
 
