@@ -715,11 +715,13 @@ sfhe_status build(const sfhe_ctx* c, int32_t n, const sfhe_matrix_view* A, const
 //    229 and 34 us against 264 for a product rounded by itself);
 //  - a unit that shares an entry 0.1 more, and the last one of an entry reads
 //    its slots, bound by latency: per slot 0.1 (one entry) to 0.3 (48 or more at
-//    once) with 512 threads, twice that with 256, 0.15 where a second CTA on the
+//    once) with 512 threads, twice that with 256, 0.1 where a second CTA on the
 //    SM hides it;
 //  - two CTAs on an SM take 1.75 times as long as one alone.
 // The estimated gains lie within 4% (one standard deviation) of the measured
-// ones, 10% where two CTAs share an SM.  One cost of 0.6 for every
+// ones.  Where two CTAs fit on an SM (N = 4096, L = 2 to 4) the chosen u of 96
+// plans is 1.6% slower in the mean than the best of their candidates (6%
+// with the units handed to one CTA on every SM first).  One cost of 0.6 for every
 // relinearisation, without playing the launch through, shared out entries of 2
 // to 9 products that ran 1.1 to 1.4 times as long for it.
 struct UnitCosts {
@@ -731,7 +733,7 @@ struct UnitCosts {
     }
     double slot(int shared) const  // entries shared out
     {
-        if (per_sm > 1) return 0.15;
+        if (per_sm > 1) return 0.1;
         return 512.0 / threads * (0.1 + 0.2 * std::min(1.0, shared / 48.0));
     }
     double slowdown(int ctas) const { return 1 + 0.75 * (ctas - 1); }
@@ -832,7 +834,11 @@ double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& 
         ev = Event{at[sm] + std::max(0.0, least) * k.slowdown(busy[sm]), order++, sm};
         return busy[sm] > 0;
     };
-    for (Cta& x : ctas) take(x);  // one CTA on every SM first
+    // neighbours of the list to the CTAs of an SM: these start together, so
+    // that a grid beyond the SMs puts long units beside long ones
+    const int grid = (int)std::min(units.size(), ctas.size());
+    for (int sm = 0; sm < k.sms; sm++)
+        for (int j = 0; j < grid / k.sms + (sm < grid % k.sms); j++) take(ctas[(size_t)j * k.sms + sm]);
     for (int sm = 0; sm < k.sms; sm++) {
         Event ev;
         if (event(sm, ev)) heap.push_back(ev);
