@@ -776,39 +776,50 @@ std::vector<Entry> units_of(const std::vector<Entry>& entries, int u)
 // The launch played through: every CTA takes the next unit when it is free,
 // the one that finishes an entry's last unit goes on to its relinearisation,
 // and the CTAs of an SM slow each other down.  Returns early, with a longer
-// time than `limit`, once it is past it.  (45 us on the host for 91 entries
-// in 168 units.)
+// time than `limit`, once it is past it.  (10 us a candidate on the
+// host for 91 entries.)
 double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& k, double limit)
 {
     struct Unit {
         int count, entry, parts;
     };
+    // longest first, entries of one length in their order (the entries come
+    // longest first): full units ahead, the rest by counting
     std::vector<Unit> units;
+    std::vector<int> at_count(u + 1, 0);
     int shared = 0;
-    for (size_t e = 0; e < entries.size(); e++) {
-        const int parts = entries[e].count <= u ? 1 : (entries[e].count + u - 1) / u;
-        for (int p = 0; p < parts; p++) units.push_back(Unit{std::min(u, entries[e].count - p * u), (int)e, parts});
+    size_t total = 0;
+    for (const Entry& e : entries) {
+        const int parts = e.count <= u ? 1 : (e.count + u - 1) / u;
         shared += parts > 1;
+        total += parts;
+        at_count[u] += parts - 1;
+        at_count[e.count - (parts - 1) * u]++;
     }
-    if (shared)  // the entries come longest first
-        std::stable_sort(units.begin(), units.end(), [](const Unit& a, const Unit& b) { return a.count > b.count; });
+    int first = 0;
+    for (int n = u; n >= 0; n--) std::swap(first, at_count[n]), first += at_count[n];
+    units.resize(total);
+    for (size_t e = 0; e < entries.size(); e++) {
+        int left = entries[e].count;
+        const int parts = left <= u ? 1 : (left + u - 1) / u;
+        for (; left > u; left -= u) units[at_count[u]++] = Unit{u, (int)e, parts};
+        units[at_count[left]++] = Unit{left, (int)e, parts};
+    }
     struct Cta {
         double left;  // of its unit, in time alone on the SM
         int unit;     // -1: none
         bool last;    // nothing follows (a whole entry's work includes its relinearisation)
     };
-    struct Event {  // an SM's next change
-        double t;
-        int order, sm;  // ties in the order of their making: units go to idle SMs first
-        bool operator>(const Event& o) const { return t != o.t ? t > o.t : order > o.order; }
-    };
     std::vector<Cta> ctas((size_t)k.sms * k.per_sm, Cta{0, -1, false});
-    std::vector<double> at(k.sms, 0);
+    std::vector<double> at(k.sms, 0), change(k.sms, 0);  // per SM: its last event and its next one
     std::vector<int> busy(k.sms, 0), finished(entries.size(), 0);
-    std::vector<Event> heap;
+    // the next events in one word each: time in 2^-18 of a product (below 2^34),
+    // then the order of their making, in which ties are taken (below 2^20: two
+    // per unit), and the SM
+    std::vector<uint64_t> heap;
     heap.reserve(k.sms);
     size_t next = 0;
-    int order = 0;
+    uint64_t order = 0;
     double end = 0;
     const double slot = k.slot(shared);
     auto take = [&](Cta& x) {
@@ -822,7 +833,7 @@ double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& 
         else if (u.count) x.left += k.relin;
     };
     // the SM's next event; false: it is idle for good
-    auto event = [&](int sm, Event& ev) {
+    auto event = [&](int sm, uint64_t& ev) {
         double least = 0;
         busy[sm] = 0;
         for (int j = 0; j < k.per_sm; j++) {
@@ -831,7 +842,8 @@ double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& 
             busy[sm]++;
             if (busy[sm] == 1 || x.left < least) least = x.left;
         }
-        ev = Event{at[sm] + std::max(0.0, least) * k.slowdown(busy[sm]), order++, sm};
+        change[sm] = at[sm] + std::max(0.0, least) * k.slowdown(busy[sm]);
+        ev = (uint64_t)(change[sm] * (1 << 18)) << 30 | order++ << 10 | (uint64_t)sm;
         return busy[sm] > 0;
     };
     // neighbours of the list to the CTAs of an SM: these start together, so
@@ -840,20 +852,21 @@ double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& 
     for (int sm = 0; sm < k.sms; sm++)
         for (int j = 0; j < grid / k.sms + (sm < grid % k.sms); j++) take(ctas[(size_t)j * k.sms + sm]);
     for (int sm = 0; sm < k.sms; sm++) {
-        Event ev;
+        uint64_t ev;
         if (event(sm, ev)) heap.push_back(ev);
     }
-    std::make_heap(heap.begin(), heap.end(), std::greater<Event>());
+    std::make_heap(heap.begin(), heap.end(), std::greater<uint64_t>());
     while (!heap.empty() && end <= limit) {
-        const Event ev = heap[0];
+        const int sm = (int)(heap[0] & 1023);
+        const double spent = (change[sm] - at[sm]) / k.slowdown(busy[sm]);
         Cta* done = nullptr;
         for (int j = 0; j < k.per_sm; j++) {
-            Cta& x = ctas[(size_t)j * k.sms + ev.sm];
+            Cta& x = ctas[(size_t)j * k.sms + sm];
             if (x.unit < 0) continue;
-            x.left -= (ev.t - at[ev.sm]) / k.slowdown(busy[ev.sm]);
+            x.left -= spent;
             if (!done || x.left < done->left) done = &x;
         }
-        at[ev.sm] = end = ev.t;
+        at[sm] = end = change[sm];
         const Unit& u = units[done->unit];
         if (!done->last && ++finished[u.entry] == u.parts) {
             done->left = k.relin + u.parts * slot;
@@ -861,17 +874,18 @@ double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& 
         } else {
             take(*done);
         }
-        Event x;
-        if (!event(ev.sm, x)) {
-            std::pop_heap(heap.begin(), heap.end(), std::greater<Event>());
+        uint64_t x;
+        if (!event(sm, x)) {
+            std::pop_heap(heap.begin(), heap.end(), std::greater<uint64_t>());
             heap.pop_back();
             continue;
         }
         // the SM's new event replaces its old one at the root
+        const size_t size = heap.size();
         size_t i = 0;
-        for (size_t c = 1; c < heap.size(); c = 2 * i + 1) {
-            if (c + 1 < heap.size() && heap[c] > heap[c + 1]) c++;
-            if (!(x > heap[c])) break;
+        for (size_t c = 1; c < size; c = 2 * i + 1) {
+            c += c + 1 < size && heap[c] > heap[c + 1];
+            if (x < heap[c]) break;
             heap[i] = heap[c];
             i = c;
         }
