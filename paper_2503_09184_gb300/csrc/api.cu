@@ -109,6 +109,7 @@ struct sfhe_plan {
     std::vector<MmDesc> mms;
     std::vector<Entry> entries;   // units: whole output entries or parts of one
     int64_t out_entries = 0;      // output entries
+    int per_sm = 0;               // CTAs on an SM, where split_entries has asked (0: not)
     int slots = 0;                // partial-sum slots of the shared-out entries
     std::vector<int> last_unit;   // with slots: per output entry its last unit, ascending
     std::vector<Entry> whole;     // with slots: the entries before they were shared out
@@ -780,6 +781,8 @@ std::vector<Entry> units_of(const std::vector<Entry>& entries, int u)
 // host for 91 entries.)
 double launch_length(const std::vector<Entry>& entries, int u, const UnitCosts& k, double limit)
 {
+    if (entries[0].count <= u && entries.size() <= (size_t)k.sms)  // an SM for every entry, the longest ends last
+        return k.work(entries[0].count) + k.relin;
     struct Unit {
         int count, entry, parts;
     };
@@ -902,6 +905,7 @@ void split_entries(const sfhe_ctx* c, sfhe_plan& P, uint32_t flags)
     for (Entry& e : P.entries) e.parts = 1, e.slot = e.first_slot = 0;
     if (!(flags & SFHE_EXEC_PERSISTENT) || P.entries.empty()) return;
     const UnitCosts costs = unit_costs(c, flags);
+    P.per_sm = costs.per_sm;
     const int grid = costs.per_sm * costs.sms, granule = costs.group;
     const int longest = P.entries[0].count;
     if (grid <= 0 || P.out_entries >= 8 * (int64_t)grid || longest <= granule) return;
@@ -974,7 +978,7 @@ Layout layout_of(const sfhe_ctx* c, const sfhe_plan& P, uint32_t flags, int* gri
     *grid_out = 0;
     *stride_out = 0;
     if (flags & SFHE_EXEC_PERSISTENT) {
-        const int per_sm = persistent_ctas_per_sm(c->rc, (flags & SFHE_EXEC_LAZY) != 0);
+        const int per_sm = P.per_sm ? P.per_sm : persistent_ctas_per_sm(c->rc, (flags & SFHE_EXEC_LAZY) != 0);
         int grid = per_sm * c->num_sms;
         grid = (int)std::min<size_t>((size_t)grid, std::max<size_t>(1, P.entries.size()));
         const size_t stride = persistent_scratch_words(c->rc);
